@@ -369,16 +369,15 @@ void build_hier(ehs_ctx* c, Hier& H, int precs, bool coef_only) {
   }
   if (nloc > 16384) throw ArgError("coarse_dd subdomains too large for dense local inverses");
   const long long N = nloc;
-  double2* M = dalloc<double2>(c, (size_t)nmat * N * 2 * N);
-  double2* fb = dalloc<double2>(c, (size_t)nmat * (N + 1));
-  int* pv = dalloc<int>(c, nmat);
+  double2* M = dalloc<double2>(c, (size_t)nmat * N * N);
+  unsigned char* iws = dalloc<unsigned char>(c, dense_invert_workspace((int)N, nmat));
   if (mgdd)
     launch_dense_assemble_sub(C.g, H.nsets, H.cdd.nsub, nloc, C.L, C.tab64, H.cdd.d_map, d_g2l, M, c->s);
   else
     launch_dense_assemble(C.g, H.nsets, C.L, C.tab64, M, c->s);
   cnt(); post();
   C.inv = dalloc<double2>(c, (size_t)nmat * N * N);
-  dense_invert((int)N, nmat, M, C.inv, fb, pv, derr, c->s); cnt(4 * N + 1); post();
+  cnt(dense_invert((int)N, nmat, M, C.inv, iws, derr, c->s)); post();
   if (precs & 2) {
     if (H.coarse_fmt == 1) {
       C.invlp = dalloc<float2>(c, (size_t)nmat * N * N);
@@ -394,7 +393,7 @@ void build_hier(ehs_ctx* c, Hier& H, int precs, bool coef_only) {
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, c->s));
   CK(cudaStreamSynchronize(c->s));
-  dfree(c, M); dfree(c, fb); dfree(c, pv); dfree(c, derr);
+  dfree(c, M); dfree(c, iws); dfree(c, derr);
   if (d_g2l) dfree(c, d_g2l);
   if (!(precs & 1)) { dfree(c, C.inv); C.inv = nullptr; }
   if (herr & EHS_DEVERR_BOX) throw CudaError("Galerkin stencil fell outside its box");

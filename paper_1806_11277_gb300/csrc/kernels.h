@@ -144,13 +144,15 @@ void launch_prolong_add(const Grid& gf, const Grid& gc, int items, const typenam
 
 // ---- coarsest level (dense FP64) ----------------------------------------
 void launch_dense_assemble(const Grid& g, int nsets, const StencilLayout& L, const double2* tab,
-                           double2* A /*[nsets][N][2N]*/, cudaStream_t s);
-void dense_invert(int N, int nsets, double2* M /*[nsets][N][2N] augmented*/, double2* inv /*[nsets][N][N]*/,
-                  double2* fbuf, int* pivbuf, int* err, cudaStream_t s);
+                           double2* A /*[nsets][N][N], zeroed*/, cudaStream_t s);
+// inv = A^{-1} for nmat matrices [N][N] (A is overwritten; ws: dense_invert_workspace bytes); returns the
+// number of launches
+size_t dense_invert_workspace(int N, int nmat);
+int dense_invert(int N, int nmat, double2* A, double2* inv, void* ws, int* err, cudaStream_t s);
 template <typename T>
 void launch_dense_apply(int N, int items, int nrhs, const double2* inv, const typename CT<T>::type* r,
                         typename CT<T>::type* x, cudaStream_t s);
-// MG-DD: local dense matrices of the coarsest-grid subdomains ([nsets*nsub][nloc][2 nloc], augmented)
+// MG-DD: local dense matrices of the coarsest-grid subdomains ([nsets*nsub][nloc][nloc], zeroed)
 void launch_dense_assemble_sub(const Grid& g, int nsets, int nsub, int nloc, const StencilLayout& L,
                                const double2* tab, const int* map, const int* g2l, double2* A, cudaStream_t s);
 // x = inv r with a low-precision inverse, FP32 accumulation; fmt 1 complex64, 2 FP16 pairs,
