@@ -475,8 +475,10 @@ void level_sweep(ehs_ctx* c, const Hier& H, int l, const typename CT<T>::type* b
       launch_st_vanka_full<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, bi, bfmt, wu, wp, 0, b, x, t, rb, var, c->s);
       launch_st_vanka_full<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, bi, bfmt, wu, wp, 1, b, t, x, rb, var, c->s);
     } else {
-      launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, wu, wp, 0, b, x, t, rb, var, c->s);
-      launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, wu, wp, 1, b, t, x, rb, var, c->s);
+      cnt(launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, wu, wp, 0, b, x, t, rb, var, c->s));
+      cnt(launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, wu, wp, 1, b, t, x, rb, var, c->s));
+      post();
+      return;
     }
     cnt(2);
   }
@@ -496,10 +498,15 @@ void autotune_rows(ehs_ctx* c, Hier& H) {
   CK(cudaEventCreate(&e1));
   // smoothed Galerkin levels, and the coarsest level when the MG-DD sweep takes residuals there
   const int ltop = H.cdd.nsub ? H.nlev : H.nlev - 1;
-  for (int l = 1; l < ltop; ++l) {
+  for (int l = 1; l < H.nlev; ++l) {
     Level& L = H.lv[l];
     int fmt = 0;
     const void* tab = tabp<T>(H, L, &fmt);
+    if (st_split(L.g, H.items, layout_variant(L.L, L.g.d), fmt)) {   // by size alone
+      L.rows_var[p] = ST_ROWS_SPLIT;
+      continue;
+    }
+    if (l >= ltop) continue;
     float best = 1e30f;
     int bestv = 0;
     for (int v = 0; v < ST_ROWS_VARIANTS; ++v) {

@@ -131,44 +131,6 @@ __global__ void k_table_cast(long long n, const double2* in, C* out) {
 // Update pass of one colour: the economic cell block (stored diagonal and
 // displacement-pressure couplings) is solved for every cell of the colour
 // from the residual r of the residual pass; xo receives the new iterate.
-// Coefficient (row A, column B, offset O) of the row at cell c from a full table
-// (slot of the layout at cell c) or a half table (compact slot at c, or its
-// mirror's at c + O; off = the linear cell offset of O), slots folded at
-// compile time.
-template <typename T, typename TT, int D, int LV, bool SYM, int A, int B, int OX, int OY, int OZ>
-__device__ __forceinline__ typename CT<T>::type tab_coef(const TT* ts, long long N, long long c, long long off) {
-  constexpr StencilLayout L = level_layout(D, LV);
-  constexpr int sl = st_slot(L, A, B, OX, OY, OZ);
-  static_assert(sl >= 0, "coefficient outside the stored box");
-  if constexpr (SYM) {
-    constexpr int q = L.pidx[A][B];
-    constexpr bool mir = half_mir_c(L, q, sl - L.p[q].base);
-    constexpr int hs = half_slot_c(L, q, sl - L.p[q].base);
-    return ldtab<T>(ts + (long long)hs * N + (mir ? c + off : c));
-  } else {
-    return ldtab<T>(ts + (long long)sl * N + c);
-  }
-}
-
-// the block coefficients of component K of the economic cell update: diagonals of the low
-// and high face, their couplings to the cell's pressure, and back
-template <typename T, typename TT, int D, int LV, bool SYM, int K>
-__device__ __forceinline__ void vupd_coefs(const TT* ts, long long N, long long c, long long sk, bool lo_ok,
-                                           bool hi_ok, typename CT<T>::type* dg, typename CT<T>::type* gr,
-                                           typename CT<T>::type* gc) {
-  constexpr int E0 = K == 0, E1 = K == 1, E2 = K == 2;
-  if (lo_ok) {
-    dg[K] = tab_coef<T, TT, D, LV, SYM, K, K, 0, 0, 0>(ts, N, c, 0);
-    gr[K] = tab_coef<T, TT, D, LV, SYM, K, D, 0, 0, 0>(ts, N, c, 0);
-    gc[K] = tab_coef<T, TT, D, LV, SYM, D, K, 0, 0, 0>(ts, N, c, 0);
-  }
-  if (hi_ok) {
-    dg[D + K] = tab_coef<T, TT, D, LV, SYM, K, K, 0, 0, 0>(ts, N, c + sk, 0);
-    gr[D + K] = tab_coef<T, TT, D, LV, SYM, K, D, -E0, -E1, -E2>(ts, N, c + sk, -sk);
-    gc[D + K] = tab_coef<T, TT, D, LV, SYM, D, K, E0, E1, E2>(ts, N, c, sk);
-  }
-}
-
 template <typename T, typename TT, int D, int LV, bool SYM>
 __global__ void __launch_bounds__(128) k_st_vupd(Grid g, int nrhs, const TT* __restrict__ tab,
                                                  T wu, T wp, int colour,
@@ -489,15 +451,23 @@ static void st_vupd_any(const Grid& g, int items, int nrhs, int v, const void* t
                                             xi, xo, s);
 }
 
-// one colour of red-black economic Vanka on a Galerkin level: residual pass
-// into rbuf (u rows of every cell, p rows of the colour), then the update pass
+// one colour of red-black economic Vanka on a Galerkin level: one launch for
+// the split launch shape of the 2D complex64 cycle, otherwise a residual pass into rbuf (u rows of every cell, p rows of the
+// colour), then the update pass
 template <typename T>
-void launch_st_vanka(const Grid& g, int items, int nrhs, const StencilLayout& L, const void* tab, int fmt,
+int launch_st_vanka(const Grid& g, int items, int nrhs, const StencilLayout& L, const void* tab, int fmt,
                      T wu, T wp, int colour, const typename CT<T>::type* b, const typename CT<T>::type* xi,
                      typename CT<T>::type* xo, typename CT<T>::type* rbuf, int var, cudaStream_t s) {
   const int v = layout_variant(L, g.d);
+  if constexpr (sizeof(T) == 4) {
+    if (var == ST_ROWS_SPLIT && g.d == 2) {
+      launch_st_colour(g, items, nrhs, v, tab, fmt, wu, wp, colour, b, xi, xo, s);
+      return 1;
+    }
+  }
   launch_st_rows<T>(g, items, nrhs, v, tab, fmt, xi, b, rbuf, 1, colour, var, s);
   st_vupd_any<T>(g, items, nrhs, v, tab, fmt, wu, wp, colour, rbuf, xi, xo, s);
+  return 2;
 }
 
 // FP64 master table -> half-precision pairs (fmt 1: FP16, 2: BF16)
@@ -621,7 +591,7 @@ void launch_st_vanka_full(const Grid& g, int items, int nrhs, const StencilLayou
   template void launch_st_resid_gather<T>(const Grid&, int, int, int, int, const int*, const StencilLayout&,   \
                                           const void*, int, const CT<T>::type*, const CT<T>::type*,          \
                                           CT<T>::type*, cudaStream_t);                                       \
-  template void launch_st_vanka<T>(const Grid&, int, int, const StencilLayout&, const void*, int, T, \
+  template int launch_st_vanka<T>(const Grid&, int, int, const StencilLayout&, const void*, int, T, \
                                    T, int, const CT<T>::type*, const CT<T>::type*, CT<T>::type*,    \
                                    CT<T>::type*, int, cudaStream_t); \
   template void launch_st_vanka_full<T>(const Grid&, int, int, const StencilLayout&, const void*, int, \

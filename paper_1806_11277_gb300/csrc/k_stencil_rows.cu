@@ -33,16 +33,17 @@ __device__ __forceinline__ void st_one_row(const Grid& g, const TT* ts, long lon
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
-__global__ void __launch_bounds__(256) k_st_rows(Grid g, int nrhs, const TT* __restrict__ tab,
+__global__ void __launch_bounds__(256) k_st_rows(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
                                                  const typename CT<T>::type* __restrict__ x,
                                                  const typename CT<T>::type* __restrict__ b,
                                                  typename CT<T>::type* __restrict__ y, int mode, int colour,
                                                  const int* __restrict__ il) {
   constexpr StencilLayout L = level_layout(D, LV);
-  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned blk = blockIdx.x / (unsigned)nit, it = blockIdx.x - blk * (unsigned)nit;
+  const long long c = (long long)blk * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int a = blockIdx.z;
-  const int item = il ? il[blockIdx.y] : blockIdx.y;
+  const int item = il ? il[it] : it;
   int i[3];
   cell_coords(g, c, i);
   if (a == D && colour >= 0 && ((i[0] + i[1] + i[2]) & 1) != colour) return;
@@ -113,30 +114,31 @@ __device__ __forceinline__ void row_acc2(typename CT<T>::type& y0, typename CT<T
         for (int ox = 0; ox < e0; ++ox) {
           const int jx = i[0] + lo0 + ox;       // neighbour of cell c; jx + 1 is the one of c + 1
           const int ti = (oz * e1 + oy) * e0 + ox;
+          // conditions on the neighbours' loads alone, as in row_acc
+          const bool in0 = rin && jx >= 0 && jx < g.n[0], in1 = rin && jx + 1 >= 0 && jx + 1 < g.n[0];
           const long long cj = c + (lo2 + oz) * sz + (lo1 + oy) * sy + (lo0 + ox);
-          Cx t0 = czero<Cx>(), t1 = czero<Cx>();
+          Cx t0 = czero<Cx>(), t1 = czero<Cx>(), x0 = czero<Cx>(), x1 = czero<Cx>();
           if constexpr (SYM) {
             // the mirror of cell c's coefficient sits at cell cj, c + 1's at cj + 1; cj is even
-            // (aligned pair load) when the x offset is even (n_x is even here)
+            // (aligned pair load) when the x offset is even (n_x is even here), and both
+            // neighbours are then inside the grid or both outside
             bool mir = false;
             const int hs = half_slot_of<D, LV, Q>(ti, mir);
-            const TT* tp = tab + (long long)hs * N + (mir ? cj : c);
-            const bool in0 = rin && jx >= 0 && jx < g.n[0], in1 = rin && jx + 1 >= 0 && jx + 1 < g.n[0];
-            if (!mir || ((lo0 + ox) & 1) == 0) {
-              if (!mir || (in0 && in1)) Pair2<TT>::ld(tp, t0, t1);
-              else {                            // a mirror cell outside the grid is not read
-                if (in0) t0 = ldtab<T>(tp);
-                if (in1) t1 = ldtab<T>(tp + 1);
-              }
+            const TT* tp = tab + (long long)hs * N;
+            if (!mir) Pair2<TT>::ld(tp + c, t0, t1);
+            else if (((lo0 + ox) & 1) == 0) {
+              if (in0) Pair2<TT>::ld(tp + cj, t0, t1);
             } else {
-              if (in0) t0 = ldtab<T>(tp);
-              if (in1) t1 = ldtab<T>(tp + 1);
+              if (in0) t0 = ldtab<T>(tp + cj);
+              if (in1) t1 = ldtab<T>(tp + cj + 1);
             }
           } else {
             Pair2<TT>::ld(tab + (long long)(base + ti) * N + c, t0, t1);
           }
-          if (rin && jx >= 0 && jx < g.n[0]) y0 = cfma(t0, __ldg(xb + cj), y0);
-          if (rin && jx + 1 >= 0 && jx + 1 < g.n[0]) y1 = cfma(t1, __ldg(xb + cj + 1), y1);
+          if (in0) x0 = __ldg(xb + cj);
+          if (in1) x1 = __ldg(xb + cj + 1);
+          y0 = cfma(t0, x0, y0);
+          y1 = cfma(t1, x1, y1);
         }
       }
     }
@@ -166,15 +168,16 @@ __device__ __forceinline__ void st_two_rows(const Grid& g, const TT* ts, long lo
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
-__global__ void k_st_rows2(Grid g, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* __restrict__ x,
+__global__ void k_st_rows2(Grid g, int nit, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* __restrict__ x,
                            const typename CT<T>::type* __restrict__ b, typename CT<T>::type* __restrict__ y,
                            int mode, int colour, const int* __restrict__ il) {
   constexpr StencilLayout L = level_layout(D, LV);
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned blk = blockIdx.x / (unsigned)nit, it = blockIdx.x - blk * (unsigned)nit;
+  const long long t = (long long)blk * blockDim.x + threadIdx.x;
   if (t >= g.ncell / 2) return;
   const long long c = 2 * t;
   const int a = blockIdx.z;
-  const int item = il ? il[blockIdx.y] : blockIdx.y;
+  const int item = il ? il[it] : it;
   int i[3];
   cell_coords(g, c, i);
   const long long N = g.ncell;
@@ -198,23 +201,26 @@ static void st_apply_t(const Grid& g, int items, int nrhs, int v, const TT* tab,
                        int var, cudaStream_t s) {
   if (var < 0 || var >= ST_ROWS_VARIANTS || (kRowsCpt[var] == 2 && (g.n[0] & 1))) var = 0;
   const int bs = kRowsBs[var];
+  // the items of a batch take turns on the same cells: their blocks run side by side, and the table
+  // entries they share come from L2 after the first
+  const int nit = (int)sel_items(items);
   if (kRowsCpt[var] == 1) {
-    const dim3 gr((unsigned)((g.ncell + bs - 1) / bs), sel_items(items), g.d + 1);
+    const dim3 gr((unsigned)((g.ncell + bs - 1) / bs) * nit, 1, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) k_st_rows<T, TT, 2, 1, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows<T, TT, 2, 2, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) k_st_rows<T, TT, 2, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else k_st_rows<T, TT, 2, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     } else if constexpr (!SYM) {
-      if (v == 1) k_st_rows<T, TT, 3, 1, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows<T, TT, 3, 2, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) k_st_rows<T, TT, 3, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else k_st_rows<T, TT, 3, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     }
   } else {
-    const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs), sel_items(items), g.d + 1);
+    const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs) * nit, 1, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) k_st_rows2<T, TT, 2, 1, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows2<T, TT, 2, 2, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) k_st_rows2<T, TT, 2, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else k_st_rows2<T, TT, 2, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     } else if constexpr (!SYM) {
-      if (v == 1) k_st_rows2<T, TT, 3, 1, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows2<T, TT, 3, 2, SYM><<<gr, bs, 0, s>>>(g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) k_st_rows2<T, TT, 3, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else k_st_rows2<T, TT, 3, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     }
   }
 }
@@ -246,6 +252,10 @@ template <typename T>
 void launch_st_rows(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt,
                     const typename CT<T>::type* x, const typename CT<T>::type* b, typename CT<T>::type* y, int mode,
                     int colour, int var, cudaStream_t s) {
+  if (var == ST_ROWS_SPLIT) {
+    launch_st_rows_split<T>(g, items, nrhs, v, tab, fmt, x, b, y, mode, colour, s);
+    return;
+  }
   st_apply_any<T>(g, items, nrhs, v, tab, fmt, x, b, y, mode, colour, var, s);
 }
 

@@ -90,12 +90,23 @@ void launch_table_cast(long long n, const double2* in, typename CT<T>::type* out
 // tab: stencil table of level-layout L in format fmt (0: complex T, full; 1: FP16
 // pairs, 2: BF16 pairs, in half storage (launch_table_half_sym) in 2D and full in
 // 3D; the half formats serve the complex64 cycle only)
-// var: residual-pass launch shape, 0 .. ST_ROWS_VARIANTS-1 (chosen by the setup autotuner)
+// var: residual-pass launch shape, 0 .. ST_ROWS_VARIANTS-1 (chosen by the setup autotuner), or ST_ROWS_SPLIT
+// where st_split holds
 #define ST_ROWS_VARIANTS 4
+#define ST_ROWS_SPLIT 4
 // layout variant of a Galerkin level: 1 = first coarse level, 2 = all coarser ones (throws otherwise)
 int layout_variant(const StencilLayout& L, int d);
 // residual pass on a Galerkin level of layout variant v (mode 0: y = K_c x, 1: y = b - K_c x;
 // colour >= 0: pressure rows of that colour only)
+// ST_ROWS_SPLIT: rows split over the warps of a block, and one colour's relaxation in one launch (2D complex64
+// cycle); k_stencil_split.cu
+bool st_split(const Grid& g, int items, int v, int fmt);
+template <typename T>
+void launch_st_rows_split(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt,
+                          const typename CT<T>::type* x, const typename CT<T>::type* b, typename CT<T>::type* y,
+                          int mode, int colour, cudaStream_t s);
+void launch_st_colour(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt, float wu, float wp, int colour,
+                      const float2* b, const float2* xi, float2* xo, cudaStream_t s);
 template <typename T>
 void launch_st_rows(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt,
                     const typename CT<T>::type* x, const typename CT<T>::type* b, typename CT<T>::type* y, int mode,
@@ -111,9 +122,9 @@ void launch_table_half(long long n, const double2* in, void* out, int fmt, cudaS
 int half_table_slots(const StencilLayout& L);
 void launch_table_half_sym(const Grid& g, int nsets, const StencilLayout& L, const double2* in, void* out, int fmt,
                            cudaStream_t s);
-// one colour of red-black Vanka on a Galerkin level; rbuf: residual scratch of x's size
+// one colour of red-black Vanka on a Galerkin level; rbuf: residual scratch of x's size; returns the launches
 template <typename T>
-void launch_st_vanka(const Grid& g, int items, int nrhs, const StencilLayout& L, const void* tab, int fmt,
+int launch_st_vanka(const Grid& g, int items, int nrhs, const StencilLayout& L, const void* tab, int fmt,
                      T wu, T wp, int colour, const typename CT<T>::type* b, const typename CT<T>::type* xi,
                      typename CT<T>::type* xo, typename CT<T>::type* rbuf, int var, cudaStream_t s);
 // full Vanka (whole cell block): setup inverses of a smoothed Galerkin level,
