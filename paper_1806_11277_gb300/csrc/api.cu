@@ -90,6 +90,8 @@ struct Hier {
   bool coef_only = false;      // only the fine coefficients were built (global problem of a DD context)
   bool fused0 = false;         // 2D complex64 cycle: fused fine-level sweep and residual + restriction
   SweepTab stab;               // setup-time tables of the fused sweep (fused0)
+  FineTab<double> ft64;        // and of the fine level's other kernels, where built (muh not null)
+  FineTab<float> ft32;
   bool persist = false;        // complex64 MG-DD coarsest solve in one persistent launch
   unsigned* pbar = nullptr;    // its grid-barrier state (2 words)
   Coef4<double>* cf64 = nullptr;
@@ -201,6 +203,31 @@ inline SelScope global_sel(ehs_ctx* c) {
 // ------------------------------------------------------------ hierarchy
 template <typename T> void autotune_rows(ehs_ctx* c, Hier& H);
 
+template <typename T> FineTab<T>& ftab(Hier& H);
+template <> FineTab<double>& ftab<double>(Hier& H) { return H.ft64; }
+template <> FineTab<float>& ftab<float>(Hier& H) { return H.ft32; }
+template <typename T> const FineTab<T>& ftab(const Hier& H) { return ftab<T>(const_cast<Hier&>(H)); }
+
+// Setup-time tables of the fine level; apply: with the plain diagonals.
+template <typename T> void build_fine_tab(ehs_ctx* c, Hier& H, bool apply) {
+  typedef typename CT<T>::type C;
+  const size_t n = (size_t)H.nsets * H.g0.ncell;
+  const int d = H.g0.d;
+  FineTab<T>& F = ftab<T>(H);
+  for (int k = 0; k < d; ++k) {
+    F.dv[k] = dalloc<C>(c, n);
+    if (apply) {
+      F.dg[k] = dalloc<C>(c, n);
+      F.rf[k] = dalloc<T>(c, n);
+    }
+  }
+  for (int k = 0; k < d * (d - 1) / 2; ++k) F.em[k] = dalloc<T>(c, n);
+  F.sinv = dalloc<C>(c, n);
+  F.muh = dalloc<T>(c, n);
+  F.kap = dalloc<T>(c, n);
+  launch_fine_tab<T>(H.g0, H.nsets, H.cf64, H.h, H.alpha, F, c->s); cnt(2); post();
+}
+
 // Builds the hierarchy of H from H.cf64.  precs: work buffers for the FP64
 // cycle (bit 0) and the complex64 cycle (bit 1).  coef_only: only the fine
 // coefficients (the global problem of a DD context, whose cycles run on the
@@ -209,6 +236,7 @@ void build_hier(ehs_ctx* c, Hier& H, int precs, bool coef_only) {
   const int d = H.g0.d;
   H.cf32 = dalloc<Coef4<float>>(c, (size_t)H.nsets * H.g0.ncell);
   launch_coef_cast<float>((long long)H.nsets * H.g0.ncell, H.cf64, H.cf32, c->s); cnt(); post();
+  if (precs & 1) build_fine_tab<double>(c, H, true);   // the FP64 operator and relaxation
   if (coef_only) {
     H.lv.resize(1);
     H.lv[0].g = H.g0;
@@ -413,6 +441,8 @@ void build_hier(ehs_ctx* c, Hier& H, int precs, bool coef_only) {
     H.stab.sinv = dalloc<float2>(c, nc);
     H.stab.vm = dalloc<float>(c, (size_t)H.nsets * sweep_table_vertices(H.g0));
     launch_sweep_tables(H.g0, H.nsets, H.cf32, H.h, H.alpha, H.stab, c->s); cnt(2); post();
+  } else if ((precs & 2) && !H.full) {
+    build_fine_tab<float>(c, H, false);
   }
   // opts.coarse_persist: the MG-DD coarsest solve of the 2D complex64 cycle as one persistent launch
   H.persist = (precs & 2) && mgdd && c->opt.coarse_persist && coarse_persist_supported(C.g, H.coarse_fmt);
@@ -440,12 +470,22 @@ template <> const void* tabp<float>(const Hier& H, const Level& L, int* fmt) {
   return L.tab32;
 }
 
+// y = K x (alpha = 0) or K_s x, or b minus it (mode 1), on the fine level of H
+template <typename T>
+void fine_apply(ehs_ctx* c, const Hier& H, double alpha, const typename CT<T>::type* x, const typename CT<T>::type* b,
+                typename CT<T>::type* y, int mode) {
+  if constexpr (sizeof(T) == 8) launch_fine_apply_tab(H.g0, H.items, H.nrhs, H.ft64, H.h, alpha, x, b, y, mode, c->s);
+  else launch_fine_apply(H.g0, H.items, H.nrhs, H.cf32, H.h, alpha, x, b, y, mode, c->s);
+  cnt(); post();
+}
+
 template <typename T>
 void level_apply(ehs_ctx* c, const Hier& H, int l, double alpha, const typename CT<T>::type* x,
                  const typename CT<T>::type* b, typename CT<T>::type* y, int mode) {
   const Level& L = H.lv[l];
   if (l == 0) {
-    launch_fine_apply<T>(L.g, H.items, H.nrhs, cfp<T>(H), H.h, alpha, x, b, y, mode, c->s);
+    fine_apply<T>(c, H, alpha, x, b, y, mode);
+    return;
   } else {
     int fmt = 0;
     const void* tab = tabp<T>(H, L, &fmt);
@@ -460,7 +500,10 @@ void level_sweep(ehs_ctx* c, const Hier& H, int l, const typename CT<T>::type* b
                  typename CT<T>::type* x, typename CT<T>::type* t) {
   const Level& L = H.lv[l];
   const T wu = (T)L.w, wp = (T)(L.w * H.wp_ratio);
-  if (l == 0) {
+  if (l == 0 && !H.full && ftab<T>(H).muh) {
+    launch_fine_vanka_tab<T>(L.g, H.items, H.nrhs, ftab<T>(H), H.h, wu, wp, 0, b, x, t, c->s);
+    launch_fine_vanka_tab<T>(L.g, H.items, H.nrhs, ftab<T>(H), H.h, wu, wp, 1, b, t, x, c->s);
+  } else if (l == 0) {
     launch_fine_vanka<T>(L.g, H.items, H.nrhs, cfp<T>(H), H.h, H.alpha, wu, wp, 0, b, x, t, c->s, H.full);
     launch_fine_vanka<T>(L.g, H.items, H.nrhs, cfp<T>(H), H.h, H.alpha, wu, wp, 1, b, t, x, c->s, H.full);
   } else {
@@ -1047,7 +1090,7 @@ ehs_status fgmres_c128(ehs_ctx* c, const double2* q, double2* u, ehs_solve_info*
         if (c->opt.precond == EHS_PRECOND_DD) dd_apply_t<double>(c, Vj, Zj);
         else cycle_rec<double>(c, c->H, 0, Vj, Zj, false);
       });
-      launch_fine_apply<double>(c->H.g0, items, c->H.nrhs, c->H.cf64, c->H.h, 0.0, Zj, nullptr, c->w, 0, s);
+      fine_apply<double>(c, c->H, 0.0, Zj, nullptr, c->w, 0);
       const int nv = j + 1;
       launch_mdot(n, items, nv, c->V, c->w, c->part, nblk, s);
       launch_reduce_parts(items, nv, nblk, c->part, c->hd, 0, s);
@@ -1055,7 +1098,7 @@ ehs_status fgmres_c128(ehs_ctx* c, const double2* q, double2* u, ehs_solve_info*
       launch_reduce_parts(items, nv, nblk, c->part, c->y, 0, s);
       launch_mupdate(n, items, nv, c->V, c->y, c->w, nullptr, nblk, 0, c->npart, s);
       launch_reduce_norm(items, nblk, c->npart, c->nrm, s);
-      cnt(7); post();
+      cnt(6); post();
       double2* ph1 = c->hstep;                         // pinned: no pageable copies
       double2* ph2 = c->hstep + (size_t)items * 12;
       double* phn = (double*)(c->hstep + (size_t)items * 24);
@@ -1069,9 +1112,9 @@ ehs_status fgmres_c128(ehs_ctx* c, const double2* q, double2* u, ehs_solve_info*
     CK(cudaMemcpyAsync(c->y, yh.data(), (size_t)items * m * sizeof(double2), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(c->kused, A.kused.data(), items * sizeof(int), cudaMemcpyHostToDevice, s));
     launch_xupdate<double2>(n, items, m, c->Z, c->y, c->kused, u, s);
-    launch_fine_apply<double>(c->H.g0, items, c->H.nrhs, c->H.cf64, c->H.h, 0.0, u, q, c->rd, 1, s);
+    fine_apply<double>(c, c->H, 0.0, u, q, c->rd, 1);
     launch_norm_part(n, items, c->rd, c->npart, nblk, s);
-    launch_reduce_norm(items, nblk, c->npart, c->nrm, s); cnt(4); post();
+    launch_reduce_norm(items, nblk, c->npart, c->nrm, s); cnt(3); post();
     sync_read(c, c->hpin, c->nrm, items * sizeof(double));
     A.end_cycle(c->hpin);
     if (A.nonfinite || A.breakdown) break;

@@ -548,17 +548,13 @@ void launch_coef_cast(long long n, const Coef4<double>* in, Coef4<T>* out, cudaS
   k_coef_cast<T><<<grid1(n, 1, 256), 256, 0, s>>>(n, in, out);
 }
 
-template <typename T>
-void launch_fine_apply(const Grid& g, int items, int nrhs, const Coef4<T>* cf, double h,
-                       double alpha, const typename CT<T>::type* x,
-                       const typename CT<T>::type* b, typename CT<T>::type* y, int mode,
-                       cudaStream_t s) {
-  const FineP<T> P = mkP<T>(h, alpha);
-  const dim3 gr((unsigned)((g.ncell + 255) / 256), sel_items(items));
-  if (g.d == 2)
-    k_fine_apply<T, 2><<<gr, 256, 0, s>>>(g, nrhs, cf, P, x, b, y, mode, g_sel.list);
-  else
-    k_fine_apply<T, 3><<<gr, 256, 0, s>>>(g, nrhs, cf, P, x, b, y, mode, g_sel.list);
+void launch_fine_apply(const Grid& g, int items, int nrhs, const Coef4<float>* cf, double h, double alpha,
+                       const float2* x, const float2* b, float2* y, int mode, cudaStream_t s) {
+  const FineP<float> P = mkP<float>(h, alpha);
+  const int bs = spread_bs(g.ncell, items, 256);
+  const dim3 gr((unsigned)((g.ncell + bs - 1) / bs), sel_items(items));
+  if (g.d == 2) k_fine_apply<float, 2><<<gr, bs, 0, s>>>(g, nrhs, cf, P, x, b, y, mode, g_sel.list);
+  else k_fine_apply<float, 3><<<gr, bs, 0, s>>>(g, nrhs, cf, P, x, b, y, mode, g_sel.list);
 }
 
 template <typename T>
@@ -575,13 +571,14 @@ void launch_fine_vanka(const Grid& g, int items, int nrhs, const Coef4<T>* cf, d
     }
   }
   const long long np = g.ncell / 2;
-  const dim3 gr((unsigned)((np + 127) / 128), sel_items(items));
+  const int bs = spread_bs(np, items, 128);
+  const dim3 gr((unsigned)((np + bs - 1) / bs), sel_items(items));
   if (g.d == 2) {
-    if (full) k_fine_vanka<T, 2, true><<<gr, 128, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
-    else k_fine_vanka<T, 2, false><<<gr, 128, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    if (full) k_fine_vanka<T, 2, true><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    else k_fine_vanka<T, 2, false><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
   } else {
-    if (full) k_fine_vanka<T, 3, true><<<gr, 128, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
-    else k_fine_vanka<T, 3, false><<<gr, 128, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    if (full) k_fine_vanka<T, 3, true><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    else k_fine_vanka<T, 3, false><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
   }
 }
 
@@ -603,9 +600,6 @@ void launch_fine_table(const Grid& g, int nsets, const Coef4<double>* cf, double
                                    const int*, const int*, const int*, const int*,                 \
                                    const Coef4<double>*, double, Coef4<T>*, cudaStream_t);         \
   template void launch_coef_cast<T>(long long, const Coef4<double>*, Coef4<T>*, cudaStream_t);     \
-  template void launch_fine_apply<T>(const Grid&, int, int, const Coef4<T>*, double,              \
-                                     double, const CT<T>::type*, const CT<T>::type*,              \
-                                     CT<T>::type*, int, cudaStream_t);                             \
   template void launch_fine_vanka<T>(const Grid&, int, int, const Coef4<T>*, double,              \
                                      double, T, T, int, const CT<T>::type*, const CT<T>::type*,    \
                                      CT<T>::type*, cudaStream_t, int);

@@ -328,12 +328,10 @@ __device__ __forceinline__ typename CT<T>::type gather_row_half(const Grid& g, c
     if (a == 0) return st_row_ct<T, TT, D, LV, SYM, 0, false, 2, 0>(g, ts, c, i, x);
     if (a == 1) return st_row_ct<T, TT, D, LV, SYM, 1, false, 2, 0>(g, ts, c, i, x);
     if (a == 2) return st_row_ct<T, TT, D, LV, SYM, 2, false, 2, 0>(g, ts, c, i, x);
-    if constexpr (D == 3) return st_row_ct<T, TT, D, LV, SYM, 3, false, 2, 0>(g, ts, c, i, x);
   } else {
     if (a == 0) return st_row_ct<T, TT, D, LV, SYM, 0, false, 2, 1>(g, ts, c, i, x);
     if (a == 1) return st_row_ct<T, TT, D, LV, SYM, 1, false, 2, 1>(g, ts, c, i, x);
     if (a == 2) return st_row_ct<T, TT, D, LV, SYM, 2, false, 2, 1>(g, ts, c, i, x);
-    if constexpr (D == 3) return st_row_ct<T, TT, D, LV, SYM, 3, false, 2, 1>(g, ts, c, i, x);
   }
   return czero<typename CT<T>::type>();
 }
@@ -358,8 +356,7 @@ __global__ void __launch_bounds__(128) k_st_resid_gather(Grid g, int nrhs, int n
   Cx v = czero<Cx>();
   const long long vo = (long long)(m * nrhs + r) * (D + 1) * N;
   if (gs >= 0) {
-    const int a = (int)(gs / N);
-    const long long c = gs % N;
+    const int a = gs / (int)N, c = gs - a * (int)N;
     constexpr int nslot = SYM ? half_base(L, L.npair) : L.nslot;
     const TT* ts = tab + (long long)m * nslot * N;
     int i[3];
@@ -419,13 +416,14 @@ template <typename T, typename TT, bool SYM>
 static void st_vupd_t(const Grid& g, int items, int nrhs, int v, const TT* tab, T wu, T wp, int colour,
                       const typename CT<T>::type* r, const typename CT<T>::type* xi, typename CT<T>::type* xo,
                       cudaStream_t s) {
-  const dim3 gu((unsigned)((g.ncell / 2 + 127) / 128), sel_items(items), 1);
+  const int bs = spread_bs(g.ncell / 2, items, 128);
+  const dim3 gu((unsigned)((g.ncell / 2 + bs - 1) / bs), sel_items(items), 1);
   if (g.d == 2) {
-    if (v == 1) k_st_vupd<T, TT, 2, 1, SYM><<<gu, 128, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
-    else k_st_vupd<T, TT, 2, 2, SYM><<<gu, 128, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
+    if (v == 1) k_st_vupd<T, TT, 2, 1, SYM><<<gu, bs, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
+    else k_st_vupd<T, TT, 2, 2, SYM><<<gu, bs, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
   } else if constexpr (!SYM) {
-    if (v == 1) k_st_vupd<T, TT, 3, 1, SYM><<<gu, 128, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
-    else k_st_vupd<T, TT, 3, 2, SYM><<<gu, 128, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
+    if (v == 1) k_st_vupd<T, TT, 3, 1, SYM><<<gu, bs, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
+    else k_st_vupd<T, TT, 3, 2, SYM><<<gu, bs, 0, s>>>(g, nrhs, tab, wu, wp, colour, r, xi, xo, g_sel.list);
   }
 }
 // dispatch on the table storage format (0: as T, full; 1: FP16 pairs, 2: BF16 pairs; T = float
@@ -483,13 +481,8 @@ static void resid_gather_t(const Grid& g, int items_l, int nrhs, int nsub, int n
                            const TT* tab, const typename CT<T>::type* x, const typename CT<T>::type* b,
                            typename CT<T>::type* out, cudaStream_t s) {
   const dim3 gr((unsigned)((nloc + 63) / 64), sel_items(items_l));   // 64 unknowns per 128-thread block
-  if (g.d == 2) {
-    if (v == 1) k_st_resid_gather<T, TT, 2, 1, SYM><<<gr, 128, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
-    else k_st_resid_gather<T, TT, 2, 2, SYM><<<gr, 128, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
-  } else if constexpr (!SYM) {
-    if (v == 1) k_st_resid_gather<T, TT, 3, 1, SYM><<<gr, 128, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
-    else k_st_resid_gather<T, TT, 3, 2, SYM><<<gr, 128, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
-  }
+  if (v == 1) k_st_resid_gather<T, TT, 2, 1, SYM><<<gr, 128, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
+  else k_st_resid_gather<T, TT, 2, 2, SYM><<<gr, 128, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
 }
 
 template <typename T>
@@ -497,18 +490,13 @@ void launch_st_resid_gather(const Grid& g, int items_l, int nrhs, int nsub, int 
                             const StencilLayout& L, const void* tab, int fmt, const typename CT<T>::type* x,
                             const typename CT<T>::type* b, typename CT<T>::type* out, cudaStream_t s) {
   const int v = layout_variant(L, g.d);
+  if (g.d == 3) return launch_st_gather3<T>(g, items_l, nrhs, nsub, nloc, map, v, tab, fmt, x, b, out, s);
   if constexpr (sizeof(T) == 4) {
-    if (fmt == 1 && g.d == 2)
+    if (fmt == 1)
       return resid_gather_t<T, __half2, true>(g, items_l, nrhs, nsub, nloc, map, v, (const __half2*)tab, x, b, out, s);
-    if (fmt == 2 && g.d == 2)
+    if (fmt == 2)
       return resid_gather_t<T, __nv_bfloat162, true>(g, items_l, nrhs, nsub, nloc, map, v,
                                                      (const __nv_bfloat162*)tab, x, b, out, s);
-    if (fmt == 1)
-      return resid_gather_t<T, __half2, false>(g, items_l, nrhs, nsub, nloc, map, v, (const __half2*)tab, x, b, out,
-                                               s);
-    if (fmt == 2)
-      return resid_gather_t<T, __nv_bfloat162, false>(g, items_l, nrhs, nsub, nloc, map, v,
-                                                      (const __nv_bfloat162*)tab, x, b, out, s);
   }
   resid_gather_t<T, typename CT<T>::type, false>(g, items_l, nrhs, nsub, nloc, map, v,
                                                  (const typename CT<T>::type*)tab, x, b, out, s);

@@ -243,6 +243,42 @@ __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int
   }
 }
 
+// 3D MG-DD colour residual at the box unknowns, as k_st_resid_gather (k_stencil.cu; 2D), with 8 warps
+// looping over the lines of 32 unknowns' rows: the unrolled rows were bound by fetching their code (one box of
+// 8^3 coarsest cells, 36 us).
+template <typename T, typename TT, int LV>
+__global__ void __launch_bounds__(256) k_st_gather3(Grid g, int nrhs, int nsub, int nloc, const int* __restrict__ map,
+                                                    const TT* __restrict__ tab,
+                                                    const typename CT<T>::type* __restrict__ x,
+                                                    const typename CT<T>::type* __restrict__ b,
+                                                    typename CT<T>::type* __restrict__ out,
+                                                    const int* __restrict__ il) {
+  typedef typename CT<T>::type Cx;
+  constexpr int nslot = level_layout(3, LV).nslot;
+  constexpr int NS = 8;
+  __shared__ Cx sp[NS][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
+  const int bl = il ? il[blockIdx.y] : blockIdx.y;
+  const int r = bl % nrhs, s = (bl / nrhs) % nsub, m = bl / (nrhs * nsub);
+  const long long N = g.ncell, vo = (long long)(m * nrhs + r) * 4 * N;
+  const int gs = e < nloc ? map[(long long)s * nloc + e] : -1;
+  Cx v = czero<Cx>();
+  if (gs >= 0) {
+    const int a = gs / (int)N, c = gs - a * (int)N;
+    int i[3];
+    cell_coords(g, c, i);
+    v = row_lines<T, TT, NS>(g, kLines[LV - 1], tab + (long long)m * nslot * N, c, i, x + vo, a, part);
+  }
+  sp[part][lane] = v;
+  __syncthreads();
+  if (part || e >= nloc) return;
+#pragma unroll
+  for (int q = 1; q < NS; ++q) v = cadd(v, sp[q][lane]);
+  if (gs >= 0) v = csub(__ldg(b + vo + gs), v);
+  out[(long long)bl * nloc + e] = v;
+}
+
 // warps per row
 template <int D> struct Ns;
 template <> struct Ns<2> { static const int rows = 4, colour = 2; };
@@ -279,6 +315,15 @@ void rows_split_d(int v, const TT* tab, const Grid& g, int items, int nrhs, cons
   } else if constexpr (!SYM) {
     if (v == 1) rows_split_t<T, TT, 3, 1, SYM>(g, items, nrhs, tab, x, b, y, mode, colour, s);
     else rows_split_t<T, TT, 3, 2, SYM>(g, items, nrhs, tab, x, b, y, mode, colour, s);
+  }
+}
+template <typename T, typename TT, bool SYM>
+void gather3_d(int v, const TT* tab, const Grid& g, int items_l, int nrhs, int nsub, int nloc, const int* map,
+               const typename CT<T>::type* x, const typename CT<T>::type* b, typename CT<T>::type* out, cudaStream_t s) {
+  if constexpr (!SYM) {
+    const dim3 gr((unsigned)((nloc + 31) / 32), sel_items(items_l));
+    if (v == 1) k_st_gather3<T, TT, 1><<<gr, 256, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
+    else k_st_gather3<T, TT, 2><<<gr, 256, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
   }
 }
 template <typename TT, int LV, bool SYM>
@@ -327,7 +372,16 @@ void launch_st_colour(const Grid& g, int items, int nrhs, int v, const void* tab
   EHS_ST_FORMATS(colour_d, g, items, nrhs, wu, wp, colour, b, xi, xo, s);
 }
 
+template <typename T>
+void launch_st_gather3(const Grid& g, int items_l, int nrhs, int nsub, int nloc, const int* map, int v, const void* tab,
+                       int fmt, const typename CT<T>::type* x, const typename CT<T>::type* b,
+                       typename CT<T>::type* out, cudaStream_t s) {
+  EHS_ST_FORMATS(gather3_d, g, items_l, nrhs, nsub, nloc, map, x, b, out, s);
+}
+
 #define INST(T)                                                                                                \
+  template void launch_st_gather3<T>(const Grid&, int, int, int, int, const int*, int, const void*, int,         \
+                                     const CT<T>::type*, const CT<T>::type*, CT<T>::type*, cudaStream_t);       \
   template void launch_st_rows_split<T>(const Grid&, int, int, int, const void*, int, const CT<T>::type*,        \
                                         const CT<T>::type*, CT<T>::type*, int, int, cudaStream_t);
 INST(float)

@@ -2,115 +2,154 @@
 // steps 2 and 4) with the bilinear staggered-grid transfer of Sec. 3: per
 // component a tensor product of 1D rules (vertex-like along the component's
 // own direction, cell-like with zero ghosts across it, cell-like with clamped
-// ghosts for p).  The 1D weights come from pw4() / pw_pair() in common.cuh
-// (exact quarters); every tap loop has a fixed trip count and is unrolled, so
-// a thread issues all of its loads back to back.  (The 2D complex64 fine
+// ghosts for p).  One thread per cell and component (blockIdx.z), so that the small
+// levels fill more of the chip and a thread's taps are few enough to be in flight
+// together; weights are integer quarters until they multiply, and real (two FMAs a tap), as
+// the FP64 form is bound by the FP64 pipe.  us with one thread for all components of a cell in
+// blocks of 128 (256 for the prolongation) -> now: see the launchers.  (The 2D complex64 fine
 // level of the cycle uses the fused kernels of k_fine_fused.cu instead.)
 #include "kernels.h"
 
 namespace ehs {
 namespace {
 
-// thread per coarse cell: fine offsets -1..2 around 2I along every direction
+// weight in quarters of fine index 2 J - 1 + t in coarse index J (t = 0..3, J a valid unknown index)
+__host__ __device__ constexpr int rw4(int kind, int t, int J, int nc) {
+  if (kind == 0) return t == 1 ? 4 : t == 3 ? 0 : 2;
+  if (t == 0) return J >= 1 ? 1 : 0;
+  if (t == 3) return J + 1 < nc ? 1 : 0;
+  return 3 + (kind == 2 && (t == 1 ? J == 0 : J + 1 == nc) ? 1 : 0);
+}
+__host__ __device__ constexpr bool rw4_agrees(int nc) {
+  for (int kind = 0; kind < 3; ++kind)
+    for (int J = kind == 0 ? 1 : 0; J < nc; ++J)
+      for (int t = 0; t < 4; ++t)
+        if (rw4(kind, t, J, nc) != pw4(kind, 2 * J - 1 + t, J, nc)) return false;
+  return true;
+}
+static_assert(rw4_agrees(1) && rw4_agrees(2) && rw4_agrees(3) && rw4_agrees(8), "restriction weights = pw4()");
+
+// q / 4 for q = 0..4, without an FP64 instruction
+template <typename T> __device__ __forceinline__ T quarters(int q);
+template <> __device__ __forceinline__ float quarters<float>(int q) { return 0.25f * (float)q; }
+template <> __device__ __forceinline__ double quarters<double>(int q) {
+  const int hi = q == 0 ? 0 : q == 1 ? 0x3fd00000 : q == 2 ? 0x3fe00000 : q == 3 ? 0x3fe80000 : 0x3ff00000;
+  return __hiloint2double(hi, 0);
+}
+// a + w v, w real
+template <typename T, typename C> __device__ __forceinline__ C rfma(T w, C v, C a) {
+  a.x = fma(w, v.x, a.x);
+  a.y = fma(w, v.y, a.y);
+  return a;
+}
+
+// thread per coarse cell and component: fine offsets -1..2 around 2 I along every direction
 template <typename T, int D>
 __global__ void k_restrict(Grid gf, Grid gc, const typename CT<T>::type* __restrict__ rf,
                            typename CT<T>::type* __restrict__ rc, const int* __restrict__ il) {
   typedef typename CT<T>::type C;
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= gc.ncell) return;
-  const int item = il ? il[blockIdx.y] : blockIdx.y;
-  const C* f = rf + (long long)item * (D + 1) * gf.ncell;
-  C* o = rc + (long long)item * (D + 1) * gc.ncell;
+  const int item = il ? il[blockIdx.y] : blockIdx.y, a = blockIdx.z;
+  const C* fa = rf + ((long long)item * (D + 1) + a) * gf.ncell;
   int I[3];
   cell_coords(gc, c, I);
-  constexpr int NZ = D == 3 ? 4 : 1;
+  C acc = czero<C>();
+  if (slot_valid(a, D, I)) {
+    int q[3][4];
 #pragma unroll
-  for (int a = 0; a <= D; ++a) {
-    C acc = czero<C>();
-    if (slot_valid(a, D, I)) {
-      T w[3][4];
+    for (int k = 0; k < D; ++k)
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
+      for (int t = 0; t < 4; ++t) q[k][t] = rw4(tkind(a, k, D), t, I[k], gc.n[k]);
+    constexpr int NZ = D == 3 ? 4 : 1;
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
-          w[k][t] = k < D ? T(0.25) * (T)pw4(tkind(a, k, D), 2 * I[k] - 1 + t, I[k], gc.n[k]) : T(t == 0);
-      const C* fa = f + (long long)a * gf.ncell;
+    for (int z = 0; z < NZ; ++z) {
+      C pl = czero<C>();                            // one plane
+      const bool zin = D < 3 || q[D - 1][z] != 0;
 #pragma unroll
-      for (int z = 0; z < NZ; ++z) {
-        const int fz = D == 3 ? 2 * I[2] - 1 + z : 0;
+      for (int y = 0; y < 4; ++y) {
+        const bool yin = zin && q[1][y] != 0;
+        const C* row = fa + ((long long)(D == 3 ? 2 * I[2] - 1 + z : 0) * gf.n[1] + (2 * I[1] - 1 + y)) * gf.n[0] +
+                       2 * I[0] - 1;
+        C rs = czero<C>();                          // one row
 #pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          const T wzy = w[2][z] * w[1][y];
-          if (wzy == T(0)) continue;
-          const long long row = ((long long)fz * gf.n[1] + (2 * I[1] - 1 + y)) * gf.n[0];
-#pragma unroll
-          for (int x = 0; x < 4; ++x)
-            if (w[0][x] != T(0)) acc = cfma(mk<T>(wzy * w[0][x], 0), __ldg(fa + row + 2 * I[0] - 1 + x), acc);
+        for (int x = 0; x < 4; ++x) {
+          C v = czero<C>();
+          if (yin && q[0][x] != 0) v = __ldg(row + x);
+          rs = rfma(quarters<T>(q[0][x]), v, rs);
         }
+        pl = rfma(quarters<T>(q[1][y]), rs, pl);
       }
+      acc = D == 3 ? rfma(quarters<T>(q[D - 1][z]), pl, acc) : pl;
     }
-    o[(long long)a * gc.ncell + c] = acc;
   }
+  rc[((long long)item * (D + 1) + a) * gc.ncell + c] = acc;
 }
 
-// thread per fine cell: at most two coarse indices per direction (pw_pair)
+// thread per fine cell and component: at most two coarse indices per direction (pw_pair)
 template <typename T, int D>
 __global__ void k_prolong_add(Grid gf, Grid gc, const typename CT<T>::type* __restrict__ ec,
                               typename CT<T>::type* __restrict__ xf, const int* __restrict__ il) {
   typedef typename CT<T>::type C;
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= gf.ncell) return;
-  const int item = il ? il[blockIdx.y] : blockIdx.y;
-  const C* e = ec + (long long)item * (D + 1) * gc.ncell;
-  C* x = xf + (long long)item * (D + 1) * gf.ncell;
+  const int item = il ? il[blockIdx.y] : blockIdx.y, a = blockIdx.z;
   int i[3];
   cell_coords(gf, c, i);
-  constexpr int NZ = D == 3 ? 2 : 1;
+  if (!slot_valid(a, D, i)) return;
+  const C* ea = ec + ((long long)item * (D + 1) + a) * gc.ncell;
+  C* x = xf + ((long long)item * (D + 1) + a) * gf.ncell + c;
+  const C old = *x;
+  int J[3][2] = {{0, 0}, {0, 0}, {0, 0}}, q[3][2];
 #pragma unroll
-  for (int a = 0; a <= D; ++a) {
-    if (!slot_valid(a, D, i)) continue;
-    int J[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-    T w[3][2] = {{T(1), T(0)}, {T(1), T(0)}, {T(1), T(0)}};
-#pragma unroll
-    for (int k = 0; k < D; ++k) pw_pair<T>(tkind(a, k, D), i[k], gc.n[k], J[k][0], w[k][0], J[k][1], w[k][1]);
-    const C* ea = e + (long long)a * gc.ncell;
-    C acc = czero<C>();
-#pragma unroll
-    for (int z = 0; z < NZ; ++z)
-#pragma unroll
-      for (int y = 0; y < 2; ++y) {
-        const T wzy = w[2][z] * w[1][y];
-        if (wzy == T(0)) continue;
-        const long long row = ((long long)J[2][z] * gc.n[1] + J[1][y]) * gc.n[0];
-#pragma unroll
-        for (int xx = 0; xx < 2; ++xx)
-          if (w[0][xx] != T(0)) acc = cfma(mk<T>(wzy * w[0][xx], 0), __ldg(ea + row + J[0][xx]), acc);
-      }
-    const long long idx = (long long)a * gf.ncell + c;
-    x[idx] = cadd(x[idx], acc);
+  for (int k = 0; k < D; ++k) {
+    float w0, w1;
+    pw_pair<float>(tkind(a, k, D), i[k], gc.n[k], J[k][0], w0, J[k][1], w1);
+    q[k][0] = (int)(4.0f * w0);
+    q[k][1] = (int)(4.0f * w1);
   }
+  constexpr int NZ = D == 3 ? 2 : 1;
+  C acc = czero<C>();
+#pragma unroll
+  for (int z = 0; z < NZ; ++z) {
+    C pl = czero<C>();
+    const bool zin = D < 3 || q[D - 1][z] != 0;
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const bool yin = zin && q[1][y] != 0;
+      const C* row = ea + ((long long)J[2][z] * gc.n[1] + J[1][y]) * gc.n[0];
+      C rs = czero<C>();
+#pragma unroll
+      for (int xx = 0; xx < 2; ++xx) {
+        C v = czero<C>();
+        if (yin && q[0][xx] != 0) v = __ldg(row + J[0][xx]);
+        rs = rfma(quarters<T>(q[0][xx]), v, rs);
+      }
+      pl = rfma(quarters<T>(q[1][y]), rs, pl);
+    }
+    acc = D == 3 ? rfma(quarters<T>(q[D - 1][z]), pl, acc) : pl;
+  }
+  *x = cadd(old, acc);
 }
-
-inline dim3 grid1(long long n, int items, int bs) { return dim3((unsigned)((n + bs - 1) / bs), items, 1); }
 
 }  // namespace
 
 template <typename T>
 void launch_restrict(const Grid& gf, const Grid& gc, int items, const typename CT<T>::type* rf,
                      typename CT<T>::type* rc, cudaStream_t s) {
-  if (gf.d == 2)
-    k_restrict<T, 2><<<grid1(gc.ncell, sel_items(items), 128), 128, 0, s>>>(gf, gc, rf, rc, g_sel.list);
-  else
-    k_restrict<T, 3><<<grid1(gc.ncell, sel_items(items), 128), 128, 0, s>>>(gf, gc, rf, rc, g_sel.list);
+  const int bs = spread_bs(gc.ncell * (gf.d + 1), items, 128);
+  const dim3 gr((unsigned)((gc.ncell + bs - 1) / bs), sel_items(items), gf.d + 1);
+  if (gf.d == 2) k_restrict<T, 2><<<gr, bs, 0, s>>>(gf, gc, rf, rc, g_sel.list);
+  else k_restrict<T, 3><<<gr, bs, 0, s>>>(gf, gc, rf, rc, g_sel.list);
 }
 
 template <typename T>
 void launch_prolong_add(const Grid& gf, const Grid& gc, int items, const typename CT<T>::type* ec,
                         typename CT<T>::type* xf, cudaStream_t s) {
-  if (gf.d == 2)
-    k_prolong_add<T, 2><<<grid1(gf.ncell, sel_items(items), 256), 256, 0, s>>>(gf, gc, ec, xf, g_sel.list);
-  else
-    k_prolong_add<T, 3><<<grid1(gf.ncell, sel_items(items), 256), 256, 0, s>>>(gf, gc, ec, xf, g_sel.list);
+  const int bs = spread_bs(gf.ncell * (gf.d + 1), items, 256);
+  const dim3 gr((unsigned)((gf.ncell + bs - 1) / bs), sel_items(items), gf.d + 1);
+  if (gf.d == 2) k_prolong_add<T, 2><<<gr, bs, 0, s>>>(gf, gc, ec, xf, g_sel.list);
+  else k_prolong_add<T, 3><<<gr, bs, 0, s>>>(gf, gc, ec, xf, g_sel.list);
 }
 
 #define INST(T)                                                                                 \

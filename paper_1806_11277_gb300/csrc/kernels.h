@@ -18,6 +18,14 @@ struct ItemSel {
 extern thread_local ItemSel g_sel;
 inline unsigned sel_items(int items) { return (unsigned)(g_sel.list ? g_sel.n : items); }
 
+// Threads per block of a one-thread-per-unit launch of n units per item: bs, halved down to one warp while
+// the blocks do not reach every SM.  A small launch is bound by what one SM does (above all by its FP64 pipe: 2
+// lanes a clock), not by the number of blocks: one FP64 colour of 64^2 cells 15.5 us on 16 SMs.
+inline int spread_bs(long long n, int items, int bs) {
+  while (bs > 32 && (n + bs - 1) / bs * (long long)sel_items(items) < 2 * 152) bs >>= 1;
+  return bs;
+}
+
 // ---- fine level (matrix-free) -------------------------------------------
 // cell coefficients from lambda, mu, rho (double, one set per medium, device)
 // and the absorbing layer; gamma = gamma_add + omega*abl_max*max_k(depth_k/L)^2;
@@ -38,18 +46,37 @@ void launch_sub_coef(const Grid& gl, const Grid& gg, int nsets_glob, int nsub,
 template <typename T>
 void launch_coef_cast(long long n, const Coef4<double>* in, Coef4<T>* out, cudaStream_t s);
 
-// y = K_s x (mode 0) or y = b - K_s x (mode 1), alpha = shift (0: unshifted)
-template <typename T>
-void launch_fine_apply(const Grid& g, int items, int nrhs, const Coef4<T>* cf, double h,
-                       double alpha, const typename CT<T>::type* x,
-                       const typename CT<T>::type* b, typename CT<T>::type* y, int mode,
-                       cudaStream_t s);
+// y = K_s x (mode 0) or y = b - K_s x (mode 1), alpha = shift (0: unshifted); complex64 (the FP64 form:
+// launch_fine_apply_tab)
+void launch_fine_apply(const Grid& g, int items, int nrhs, const Coef4<float>* cf, double h, double alpha,
+                       const float2* x, const float2* b, float2* y, int mode, cudaStream_t s);
 // one colour of red-black economic cell-wise relaxation: xo = xi + W B^{-1}(b - K_s xi)
 template <typename T>
 void launch_fine_vanka(const Grid& g, int items, int nrhs, const Coef4<T>* cf, double h,
                        double alpha, T wu, T wp, int colour,
                        const typename CT<T>::type* b, const typename CT<T>::type* xi,
                        typename CT<T>::type* xo, cudaStream_t s, int full = 0);
+// Setup-time tables of the fine level and the kernels that read them (k_fine_tab.cu): inverse and plain
+// (dg, rf; null where the operator is not applied from them) face-row diagonals, inverse Schur complements, mu / h^2,
+// 1 / (lambda + mu), edge means; [nsets][ncell] each
+template <typename T> struct FineTab {
+  typename CT<T>::type* dv[3] = {nullptr, nullptr, nullptr};
+  typename CT<T>::type* dg[3] = {nullptr, nullptr, nullptr};
+  T* rf[3] = {nullptr, nullptr, nullptr};
+  typename CT<T>::type* sinv = nullptr;
+  T* muh = nullptr;
+  T* kap = nullptr;
+  T* em[3] = {nullptr, nullptr, nullptr};
+};
+template <typename T>
+void launch_fine_tab(const Grid& g, int nsets, const Coef4<double>* cf, double h, double alpha, const FineTab<T>& F,
+                     cudaStream_t s);
+template <typename T>
+void launch_fine_vanka_tab(const Grid& g, int items, int nrhs, const FineTab<T>& F, double h, T wu, T wp, int colour,
+                           const typename CT<T>::type* b, const typename CT<T>::type* xi, typename CT<T>::type* xo,
+                           cudaStream_t s);
+void launch_fine_apply_tab(const Grid& g, int items, int nrhs, const FineTab<double>& F, double h, double alpha,
+                           const double2* x, const double2* b, double2* y, int mode, cudaStream_t s);
 // Fused fine-level kernels of the 2D complex64 cycle (economic block), for grids
 // that split into their tiles (fine_tiles_fit).  One whole red-black sweep:
 // xo = sweep(x_in), x_in = (xi or 0) + (P ec if ec), xo != xi; ec: coarse
@@ -105,6 +132,10 @@ template <typename T>
 void launch_st_rows_split(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt,
                           const typename CT<T>::type* x, const typename CT<T>::type* b, typename CT<T>::type* y,
                           int mode, int colour, cudaStream_t s);
+template <typename T>   // the 3D form of launch_st_resid_gather
+void launch_st_gather3(const Grid& g, int items_l, int nrhs, int nsub, int nloc, const int* map, int v, const void* tab,
+                       int fmt, const typename CT<T>::type* x, const typename CT<T>::type* b,
+                       typename CT<T>::type* out, cudaStream_t s);
 void launch_st_colour(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt, float wu, float wp, int colour,
                       const float2* b, const float2* xi, float2* xo, cudaStream_t s);
 template <typename T>
