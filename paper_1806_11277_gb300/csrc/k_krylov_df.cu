@@ -775,20 +775,60 @@ __global__ void k_fine_apply_df(Grid g, int nrhs, const Coef4df* __restrict__ cf
   dfc_st(y + vo + (long long)D * N + c, r);
 }
 
-// coarsest: x = Ainv r with Ainv in complex df64, r and x complex64; one warp per row
-__global__ void k_dense_apply_df(int N, int nrhs, const float4* __restrict__ inv,
-                                 const float2* __restrict__ r, float2* __restrict__ x,
-                                 const int* __restrict__ il) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// coarsest: x = Ainv r with Ainv in complex df64, r and x complex64.  A warp takes two rows, four columns of each
+// lane in flight at a time (8 matrix loads of 16 B; one warp per row with one load at a time and a renormalised
+// df64 multiply-add per entry: 61 us for one 3225^2 matrix, 166 MB, of which the arithmetic alone is 20).  Sums are
+// compensated Dot2 (dacc2 in df64.cuh) with the entry's high and low parts against the single-precision r.
+__device__ __forceinline__ void dacc2_fmaf(dacc2& a, float2 xh, float2 xl, float2 y) {
+  const float2 p = __fmul2_rn(xh, y);
+  const float2 pe = __ffma2_rn(xl, y, __ffma2_rn(xh, y, f2neg(p)));
+  const float2 t = __fadd2_rn(a.s, p);
+  const float2 bb = __fadd2_rn(t, f2neg(a.s));
+  const float2 sg = __fadd2_rn(__fadd2_rn(a.s, f2neg(__fadd2_rn(t, f2neg(bb)))), __fadd2_rn(p, f2neg(bb)));
+  a.s = t;
+  a.c = __fadd2_rn(a.c, __fadd2_rn(sg, pe));
+}
+__global__ void __launch_bounds__(256) k_dense_apply_df(int N, int nrhs, const float4* __restrict__ inv,
+                                                        const float2* __restrict__ r, float2* __restrict__ x,
+                                                        const int* __restrict__ il) {
+  constexpr int R = 2, U = 4;
+  const int row0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * R;
   const int lane = threadIdx.x & 31;
   const int item = il ? il[blockIdx.y] : blockIdx.y;
-  if (warp >= N) return;
-  const float4* row = inv + ((long long)(item / nrhs) * N + warp) * N;
+  if (row0 >= N) return;
+  const float4* m[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) m[k] = inv + ((long long)(item / nrhs) * N + min(row0 + k, N - 1)) * N;
   const float2* rv = r + (long long)item * N;
-  dfc acc = dfc_zero();
-  for (int j = lane; j < N; j += 32) acc = dfc_add(acc, dfc_mulf(dfc_ld(row + j), __ldg(rv + j)));
-  acc = warp_sum_df(acc);
-  if (lane == 0) x[(long long)item * N + warp] = dfc_to_f2(acc);
+  dacc2 acc[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) acc[k] = dacc2_zero();
+  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int j0 = lane; j0 < N; j0 += 32 * U) {
+    float4 a[R][U];
+    float2 b[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 32 * u;
+      const bool in = j < N;
+#pragma unroll
+      for (int k = 0; k < R; ++k) a[k][u] = in ? __ldg(m[k] + j) : z4;
+      b[u] = in ? __ldg(rv + j) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        const float4 v = a[k][u];   // the storage order of dfc_st
+        dacc2_fmaf(acc[k], make_float2(v.x, v.y), make_float2(v.z, v.w), make_float2(b[u].x, b[u].x));
+        dacc2_fmaf(acc[k], make_float2(v.y, v.x), make_float2(v.w, v.z), make_float2(-b[u].y, b[u].y));
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const dfc s = warp_sum_df(dacc2_val(acc[k]));
+    if (lane == 0 && row0 + k < N) x[(long long)item * N + row0 + k] = dfc_to_f2(s);
+  }
 }
 
 inline unsigned nb(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
@@ -937,8 +977,9 @@ void launch_fine_apply_df(const Grid& g, int items, int nrhs, const void* cf, do
 }
 void launch_dense_apply_df(int N, int items, int nrhs, const float4* inv, const float2* r, float2* x,
                            cudaStream_t s) {
-  const int wpb = 8;
-  k_dense_apply_df<<<dim3((N + wpb - 1) / wpb, sel_items(items)), 32 * wpb, 0, s>>>(N, nrhs, inv, r, x, g_sel.list);
+  const int bs = spread_bs((long long)(N + 1) / 2 * 32, items, 256);   // a warp per two rows
+  const int rpb = bs / 32 * 2;
+  k_dense_apply_df<<<dim3((N + rpb - 1) / rpb, sel_items(items)), bs, 0, s>>>(N, nrhs, inv, r, x, g_sel.list);
 }
 
 }  // namespace ehs
