@@ -18,6 +18,7 @@
 namespace ehs {
 std::atomic<long long> g_launches{0};
 thread_local ItemSel g_sel;
+thread_local bool g_pdl = true;
 }
 
 using namespace ehs;
@@ -56,6 +57,7 @@ struct Level {
   void* invlp = nullptr;      // coarsest inverse in complex64 / FP16 / BF16 pairs (coarse_fmt 1..3)
   void* binv[2] = {nullptr, nullptr};  // full Vanka block inverses [prec: 0 double2, 1 float2 or half pairs]
   void* ws[2][4] = {{nullptr}};  // [prec: 0 double, 1 float][b, x, t, r]
+  void* vt[2] = {nullptr, nullptr};   // economic cell blocks of a smoothed Galerkin level (launch_vupd_tab)
   int rows_var[2] = {0, 0};      // residual-pass launch shape per precision (setup autotuner)
   double w = 0.5;
 };
@@ -202,6 +204,7 @@ inline SelScope global_sel(ehs_ctx* c) {
 
 // ------------------------------------------------------------ hierarchy
 template <typename T> void autotune_rows(ehs_ctx* c, Hier& H);
+template <typename T> void build_vupd_tabs(ehs_ctx* c, Hier& H);
 
 template <typename T> FineTab<T>& ftab(Hier& H);
 template <> FineTab<double>& ftab<double>(Hier& H) { return H.ft64; }
@@ -426,6 +429,8 @@ void build_hier(ehs_ctx* c, Hier& H, int precs, bool coef_only) {
   if (!(precs & 1)) { dfree(c, C.inv); C.inv = nullptr; }
   if (herr & EHS_DEVERR_BOX) throw CudaError("Galerkin stencil fell outside its box");
   if (herr & EHS_DEVERR_SINGULAR) throw ArgError("coarsest Galerkin operator is singular");
+  if (precs & 2) build_vupd_tabs<float>(c, H);
+  if (precs & 1) build_vupd_tabs<double>(c, H);
   if (precs & 2) autotune_rows<float>(c, H);
   if (precs & 1) autotune_rows<double>(c, H);
   // the fused fine-level kernels serve the economic 2D complex64 cycle on grids that split into
@@ -518,14 +523,28 @@ void level_sweep(ehs_ctx* c, const Hier& H, int l, const typename CT<T>::type* b
       launch_st_vanka_full<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, bi, bfmt, wu, wp, 0, b, x, t, rb, var, c->s);
       launch_st_vanka_full<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, bi, bfmt, wu, wp, 1, b, t, x, rb, var, c->s);
     } else {
-      cnt(launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, wu, wp, 0, b, x, t, rb, var, c->s));
-      cnt(launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, wu, wp, 1, b, t, x, rb, var, c->s));
+      const C* vt = (const C*)L.vt[PT<T>::i];
+      cnt(launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, vt, wu, wp, 0, b, x, t, rb, var, c->s));
+      cnt(launch_st_vanka<T>(L.g, H.items, H.nrhs, L.L, tab, fmt, vt, wu, wp, 1, b, t, x, rb, var, c->s));
       post();
       return;
     }
     cnt(2);
   }
   cnt(2); post();
+}
+
+// Setup-time tables of the economic cell blocks of every smoothed Galerkin level.
+template <typename T> void build_vupd_tabs(ehs_ctx* c, Hier& H) {
+  typedef typename CT<T>::type C;
+  for (int l = 1; l + 1 < H.nlev && !H.full; ++l) {
+    Level& L = H.lv[l];
+    int fmt = 0;
+    const void* tab = tabp<T>(H, L, &fmt);
+    C* vt = dalloc<C>(c, (size_t)H.nsets * (L.g.d + 1) * L.g.ncell);
+    launch_vupd_tab<T>(L.g, H.nsets, L.L, tab, fmt, vt, c->s); cnt(); post();
+    L.vt[PT<T>::i] = vt;
+  }
 }
 
 // Setup autotuner: times every residual-pass launch shape of each smoothed
@@ -1029,10 +1048,23 @@ void sync_read(ehs_ctx* c, void* host, const void* dev, size_t bytes) {
   CK(cudaStreamSynchronize(c->s));
 }
 
+// Plain launches (no programmatic dependence) in its scope when off.
+struct PdlScope {
+  bool old;
+  explicit PdlScope(bool on) : old(g_pdl) { g_pdl = on; }
+  ~PdlScope() { g_pdl = old; }
+};
+
 // Runs body() (a fixed sequence of launches on c->s) directly, or replays it
-// from a CUDA graph captured on the first call for slot j.
+// from a CUDA graph captured on the first call for slot j.  Since the launches wait for
+// one another on the device (launch_pdl), a graph only pays where the host could not launch
+// fast enough: a batch of up to 64 K cells (64^2 FP64: 2.67 ms a solve replayed, 2.76
+// launched; two media of 512^2: 14.27 replayed, 13.94 launched) and the hundreds of launches of
+// a DD application, there with plain edges (launch_pdl).
 template <typename F> void graphed(ehs_ctx* c, int j, F body) {
-  if (!c->use_graphs) { body(); return; }
+  const bool dd = c->opt.precond == EHS_PRECOND_DD;
+  if (!c->use_graphs || (!dd && (long long)c->H.items * c->H.g0.ncell > 65536)) { body(); return; }
+  const PdlScope pdl(!dd);
   if (c->pg[j] && c->pg_ver[j] != c->act_ver) {   // the active item set changed
     cudaGraphExecDestroy(c->pg[j]);
     c->pg[j] = nullptr;
@@ -1227,6 +1259,7 @@ ehs_status fgmres(ehs_ctx* c, const double2* q, double2* u, ehs_solve_info* info
 }
 
 __global__ void k_conj(long long n, double2* v) {
+  pdl_enter();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < n) v[e].y = -v[e].y;
 }
@@ -1260,9 +1293,9 @@ ehs_status solve_common(ehs_ctx* c, const void* qin, void* uout, ehs_solve_info*
   }
   if (!udev) u = c->ud;
   const long long n = (long long)c->H.items * c->n0;
-  if (adjoint) { k_conj<<<(unsigned)((n + 255) / 256), 256, 0, c->s>>>(n, c->qd); cnt(); post(); }
+  if (adjoint) { launch_pdl((unsigned)((n + 255) / 256), 256, 0, c->s, k_conj, n, c->qd); cnt(); post(); }
   ehs_status st = fgmres(c, q, u, info);
-  if (adjoint) { k_conj<<<(unsigned)((n + 255) / 256), 256, 0, c->s>>>(n, u); cnt(); post(); }
+  if (adjoint) { launch_pdl((unsigned)((n + 255) / 256), 256, 0, c->s, k_conj, n, u); cnt(); post(); }
   if (!udev) {
     CK(cudaMemcpyAsync(uout, u, bytes, cudaMemcpyDeviceToHost, c->s));
     CK(cudaStreamSynchronize(c->s));

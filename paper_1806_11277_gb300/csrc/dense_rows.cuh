@@ -26,7 +26,7 @@ __device__ __forceinline__ float2 ldlp(const __nv_bfloat162* p) { return __bfloa
 // correction into the coarsest vector.
 template <typename TI, bool RCG = false, bool SCATTER = false>
 __device__ __forceinline__ void dense_rows4(int N, int n, int row0, const TI* __restrict__ mat,
-                                            const float2* __restrict__ r, float2* __restrict__ x,
+                                            const float2* r, float2* __restrict__ x,
                                             const int* __restrict__ map = nullptr, float2* xg = nullptr) {
   constexpr int E = 16 / (int)sizeof(TI);
   constexpr int R = 4;
@@ -45,7 +45,7 @@ __device__ __forceinline__ void dense_rows4(int N, int n, int row0, const TI* __
     for (int k = 0; k < R; ++k) a[k].u = __ldg(m0 + (long long)k * qs + q);
 #pragma unroll
     for (int e = 0; e < E; e += 2) {
-      const float4 b = RCG ? __ldcg(rv + (q * E + e) / 2) : __ldg(rv + (q * E + e) / 2);
+      const float4 b = RCG ? __ldcg(rv + (q * E + e) / 2) : *(rv + (q * E + e) / 2);
 #pragma unroll
       for (int k = 0; k < R; ++k) {
         const float2 c0 = ldlp(&a[k].t[e]), c1 = ldlp(&a[k].t[e + 1]);

@@ -10,7 +10,8 @@ namespace {
 
 template <typename C>
 __global__ void k_dd_gather(long long nl, int nsub, int nrhs, long long ng, const int* __restrict__ map,
-                            const C* __restrict__ res, C* __restrict__ out, const int* __restrict__ il) {
+                            const C* res, C* __restrict__ out, const int* il) {
+  pdl_enter();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nl) return;
   const int bl = il ? il[blockIdx.y] : blockIdx.y;
@@ -23,7 +24,8 @@ __global__ void k_dd_gather(long long nl, int nsub, int nrhs, long long ng, cons
 
 template <typename C>
 __global__ void k_dd_scatter(long long nl, int nsub, int nrhs, long long ng, const int* __restrict__ map,
-                             const C* __restrict__ xs, C* __restrict__ x, const int* __restrict__ il) {
+                             const C* xs, C* __restrict__ x, const int* il) {
+  pdl_enter();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nl) return;
   const int bl = il ? il[blockIdx.y] : blockIdx.y;
@@ -38,6 +40,7 @@ __global__ void k_dd_scatter(long long nl, int nsub, int nrhs, long long ng, con
 
 __global__ void k_expand_items(const int* __restrict__ list, int nact, int nrhs, int nsub,
                                const int* __restrict__ subs, int ncs, int* __restrict__ out) {
+  pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nact * ncs) return;
   const int j = t / ncs, q = t % ncs;
@@ -51,19 +54,19 @@ __global__ void k_expand_items(const int* __restrict__ list, int nact, int nrhs,
 template <typename T>
 void launch_dd_gather(long long nl, int items_l, int nsub, int nrhs, long long ng, const int* map,
                       const typename CT<T>::type* res, typename CT<T>::type* out, cudaStream_t s) {
-  k_dd_gather<<<dim3((unsigned)((nl + 255) / 256), sel_items(items_l)), 256, 0, s>>>(nl, nsub, nrhs, ng, map, res, out,
+  launch_pdl(dim3((unsigned)((nl + 255) / 256), sel_items(items_l)), 256, 0, s, k_dd_gather<typename CT<T>::type>, nl, nsub, nrhs, ng, map, res, out,
                                                                                    g_sel.list);
 }
 template <typename T>
 void launch_dd_scatter(long long nl, int items_l, int nsub, int nrhs, long long ng, const int* map,
                        const typename CT<T>::type* xs, typename CT<T>::type* x, cudaStream_t s) {
-  k_dd_scatter<<<dim3((unsigned)((nl + 255) / 256), sel_items(items_l)), 256, 0, s>>>(nl, nsub, nrhs, ng, map, xs, x,
+  launch_pdl(dim3((unsigned)((nl + 255) / 256), sel_items(items_l)), 256, 0, s, k_dd_scatter<typename CT<T>::type>, nl, nsub, nrhs, ng, map, xs, x,
                                                                                     g_sel.list);
 }
 void launch_expand_items(const int* list, int nact, int nrhs, int nsub, const int* subs, int ncs, int* out,
                          cudaStream_t s) {
   const int n = nact * ncs;
-  k_expand_items<<<(n + 127) / 128, 128, 0, s>>>(list, nact, nrhs, nsub, subs, ncs, out);
+  launch_pdl((n + 127) / 128, 128, 0, s, k_expand_items, list, nact, nrhs, nsub, subs, ncs, out);
 }
 
 template void launch_dd_gather<float>(long long, int, int, int, long long, const int*, const float2*, float2*, cudaStream_t);

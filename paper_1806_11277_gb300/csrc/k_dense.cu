@@ -51,8 +51,9 @@ __global__ void k_dense_assemble(Grid g, StencilLayout L, const double2* __restr
 // x = Ainv r, one warp per dense row; input/output in the working precision
 template <typename T>
 __global__ void k_dense_apply(int N, int nrhs, const double2* __restrict__ inv,
-                              const typename CT<T>::type* __restrict__ r,
-                              typename CT<T>::type* __restrict__ x, const int* __restrict__ il) {
+                              const typename CT<T>::type* r,
+                              typename CT<T>::type* __restrict__ x, const int* il) {
+  pdl_enter();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int item = il ? il[blockIdx.y] : blockIdx.y;
@@ -62,7 +63,7 @@ __global__ void k_dense_apply(int N, int nrhs, const double2* __restrict__ inv,
   double sx = 0.0, sy = 0.0;
   for (int j = lane; j < N; j += 32) {
     const double2 a = __ldg(row + j);
-    const typename CT<T>::type b = __ldg(rv + j);
+    const typename CT<T>::type b = *(rv + j);
     sx = fma(a.x, (double)b.x, fma(-a.y, (double)b.y, sx));
     sy = fma(a.x, (double)b.y, fma(a.y, (double)b.x, sy));
   }
@@ -122,8 +123,9 @@ __global__ void k_dense_assemble_sub(Grid g, StencilLayout L, const double2* __r
 // accumulation); one warp per row, four independent loads in flight per lane
 
 template <typename TI>
-__global__ void k_dense_apply_lp(int N, int nrhs, const TI* __restrict__ inv, const float2* __restrict__ r,
-                                 float2* __restrict__ x, const int* __restrict__ il) {
+__global__ void k_dense_apply_lp(int N, int nrhs, const TI* __restrict__ inv, const float2* r,
+                                 float2* __restrict__ x, const int* il) {
+  pdl_enter();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int item = il ? il[blockIdx.y] : blockIdx.y;
@@ -134,14 +136,14 @@ __global__ void k_dense_apply_lp(int N, int nrhs, const TI* __restrict__ inv, co
   int j = lane;
   for (; j + 96 < N; j += 128) {
     const float2 a0 = ldlp(row + j), a1 = ldlp(row + j + 32), a2 = ldlp(row + j + 64), a3 = ldlp(row + j + 96);
-    const float2 b0 = __ldg(rv + j), b1 = __ldg(rv + j + 32), b2 = __ldg(rv + j + 64), b3 = __ldg(rv + j + 96);
+    const float2 b0 = *(rv + j), b1 = *(rv + j + 32), b2 = *(rv + j + 64), b3 = *(rv + j + 96);
     sx0 = fmaf(a0.x, b0.x, fmaf(-a0.y, b0.y, sx0)); sy0 = fmaf(a0.x, b0.y, fmaf(a0.y, b0.x, sy0));
     sx1 = fmaf(a1.x, b1.x, fmaf(-a1.y, b1.y, sx1)); sy1 = fmaf(a1.x, b1.y, fmaf(a1.y, b1.x, sy1));
     sx0 = fmaf(a2.x, b2.x, fmaf(-a2.y, b2.y, sx0)); sy0 = fmaf(a2.x, b2.y, fmaf(a2.y, b2.x, sy0));
     sx1 = fmaf(a3.x, b3.x, fmaf(-a3.y, b3.y, sx1)); sy1 = fmaf(a3.x, b3.y, fmaf(a3.y, b3.x, sy1));
   }
   for (; j < N; j += 32) {
-    const float2 a = ldlp(row + j), b = __ldg(rv + j);
+    const float2 a = ldlp(row + j), b = *(rv + j);
     sx0 = fmaf(a.x, b.x, fmaf(-a.y, b.y, sx0)); sy0 = fmaf(a.x, b.y, fmaf(a.y, b.x, sy0));
   }
   float sx = sx0 + sx1, sy = sy0 + sy1;
@@ -157,8 +159,9 @@ __global__ void k_dense_apply_lp(int N, int nrhs, const TI* __restrict__ inv, co
 // sizes[set % nsub]; groups of rows at or beyond it are skipped.
 template <typename TI>
 __global__ void __launch_bounds__(256) k_dense_apply_v(int N, int nrhs, int nsub, const int* __restrict__ sizes,
-                                                       const TI* __restrict__ inv, const float2* __restrict__ r,
-                                                       float2* __restrict__ x, const int* __restrict__ il) {
+                                                       const TI* __restrict__ inv, const float2* r,
+                                                       float2* __restrict__ x, const int* il) {
+  pdl_enter();
   const int row0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4;
   const int item = il ? il[blockIdx.y] : blockIdx.y;
   const int set = item / nrhs;
@@ -167,15 +170,36 @@ __global__ void __launch_bounds__(256) k_dense_apply_v(int N, int nrhs, int nsub
   dense_rows4<TI>(N, n, row0, inv + (long long)set * N * N, r + (long long)item * N, x + (long long)item * N);
 }
 
+// The inverses are setup-time data, so a block that is resident while its predecessor still runs (launch_pdl: the
+// colour's residual gather, latency-bound and nearly idle on HBM) asks for the first `pre` bytes of each of its
+// rows before it waits.  The budget is 64 MB a launch over all its warps: half of L2, about what HBM delivers in
+// the time of a gather.  In the 512^2 cycle (one medium, four
+// colours) with the other kernels' early loads: 245 -> 239 us.
+__device__ __forceinline__ void prefetch_rows(const void* row, long long row_bytes, int rows, int pre) {
+  const int lane = threadIdx.x & 31;
+  if (lane < rows && pre > 0) {
+    const char* p = (const char*)row + lane * row_bytes;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(pre) : "memory");
+  }
+}
+
 // The MG-DD form that also scatters: sub-item = ((m * nsub) + s) * nrhs + r, its four results
 // added to the coarsest vector xg of item m * nrhs + r at the subdomain's unknowns map[s][row]
 // (subdomains of one colour are disjoint, so no two threads add to the same entry).
 template <typename TI>
 __global__ void __launch_bounds__(256) k_dense_apply_vs(int N, int nrhs, int nsub, const int* __restrict__ sizes,
-                                                        const TI* __restrict__ inv, const float2* __restrict__ r,
+                                                        const TI* __restrict__ inv, const float2* r,
                                                         const int* __restrict__ map, long long NG, float2* xg,
-                                                        const int* __restrict__ il) {
+                                                        const int* il, int pre) {
+  pdl_trigger();
   const int row0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4;
+  if (row0 < N) {
+    // il may be from the launch before this one and not yet written: then it holds older items, and what is
+    // asked for early is of no use, no more
+    const int early = il ? il[blockIdx.y] : blockIdx.y;
+    prefetch_rows(inv + ((long long)(early / nrhs) * N + row0) * N, (long long)N * sizeof(TI), 4, pre);
+  }
+  pdl_wait();
   const int item = il ? il[blockIdx.y] : blockIdx.y;
   const int set = item / nrhs, sub = set % nsub;
   const int n = sizes[sub];
@@ -193,15 +217,17 @@ bool launch_dense_apply_scatter(int N, int items, int nrhs, int nsub, const int*
   const int E = fmt >= 2 ? 4 : 2;
   if (N % 4 != 0 || N % E != 0 || !sizes) return false;
   const dim3 gv((N / 4 + wpb - 1) / wpb, sel_items(items));   // a warp per 4 rows
+  const long long row = (long long)N * (fmt >= 2 ? 4 : 8), share = (64ll << 20) / ((long long)gv.x * gv.y * wpb * 4);
+  const int pre = (int)((share < row ? share : row) / 16 * 16);
   if (fmt == 2)
-    k_dense_apply_vs<__half2><<<gv, 32 * wpb, 0, s>>>(N, nrhs, nsub, sizes, (const __half2*)inv, r, map, NG, xg,
-                                                       g_sel.list);
+    launch_pdl(gv, 32 * wpb, 0, s, k_dense_apply_vs<__half2>, N, nrhs, nsub, sizes, (const __half2*)inv, r, map, NG, xg,
+                                                       g_sel.list, pre);
   else if (fmt == 3)
-    k_dense_apply_vs<__nv_bfloat162><<<gv, 32 * wpb, 0, s>>>(N, nrhs, nsub, sizes, (const __nv_bfloat162*)inv, r, map,
-                                                              NG, xg, g_sel.list);
+    launch_pdl(gv, 32 * wpb, 0, s, k_dense_apply_vs<__nv_bfloat162>, N, nrhs, nsub, sizes, (const __nv_bfloat162*)inv, r, map,
+                                                              NG, xg, g_sel.list, pre);
   else
-    k_dense_apply_vs<float2><<<gv, 32 * wpb, 0, s>>>(N, nrhs, nsub, sizes, (const float2*)inv, r, map, NG, xg,
-                                                      g_sel.list);
+    launch_pdl(gv, 32 * wpb, 0, s, k_dense_apply_vs<float2>, N, nrhs, nsub, sizes, (const float2*)inv, r, map, NG, xg,
+                                                      g_sel.list, pre);
   return true;
 }
 
@@ -218,7 +244,7 @@ void launch_dense_apply(int N, int items, int nrhs, const double2* inv, const ty
                         typename CT<T>::type* x, cudaStream_t s) {
   const int wpb = 8;
   dim3 grid((N + wpb - 1) / wpb, sel_items(items));
-  k_dense_apply<T><<<grid, 32 * wpb, 0, s>>>(N, nrhs, inv, r, x, g_sel.list);
+  launch_pdl(grid, 32 * wpb, 0, s, k_dense_apply<T>, N, nrhs, inv, r, x, g_sel.list);
 }
 
 void launch_dense_assemble_sub(const Grid& g, int nsets, int nsub, int nloc, const StencilLayout& L,
@@ -236,20 +262,20 @@ void launch_dense_apply_lp(int N, int items, int nrhs, int nsub, const int* size
   if (N % 4 == 0 && N % E == 0) {
     const dim3 gv((N / 4 + wpb - 1) / wpb, sel_items(items));   // a warp per 4 rows
     if (fmt == 2)
-      k_dense_apply_v<__half2><<<gv, 32 * wpb, 0, s>>>(N, nrhs, nsub, sizes, (const __half2*)inv, r, x, g_sel.list);
+      launch_pdl(gv, 32 * wpb, 0, s, k_dense_apply_v<__half2>, N, nrhs, nsub, sizes, (const __half2*)inv, r, x, g_sel.list);
     else if (fmt == 3)
-      k_dense_apply_v<__nv_bfloat162><<<gv, 32 * wpb, 0, s>>>(N, nrhs, nsub, sizes, (const __nv_bfloat162*)inv, r, x,
+      launch_pdl(gv, 32 * wpb, 0, s, k_dense_apply_v<__nv_bfloat162>, N, nrhs, nsub, sizes, (const __nv_bfloat162*)inv, r, x,
                                                               g_sel.list);
     else
-      k_dense_apply_v<float2><<<gv, 32 * wpb, 0, s>>>(N, nrhs, nsub, sizes, (const float2*)inv, r, x, g_sel.list);
+      launch_pdl(gv, 32 * wpb, 0, s, k_dense_apply_v<float2>, N, nrhs, nsub, sizes, (const float2*)inv, r, x, g_sel.list);
     return;
   }
   if (fmt == 2)
-    k_dense_apply_lp<__half2><<<grid, 32 * wpb, 0, s>>>(N, nrhs, (const __half2*)inv, r, x, g_sel.list);
+    launch_pdl(grid, 32 * wpb, 0, s, k_dense_apply_lp<__half2>, N, nrhs, (const __half2*)inv, r, x, g_sel.list);
   else if (fmt == 3)
-    k_dense_apply_lp<__nv_bfloat162><<<grid, 32 * wpb, 0, s>>>(N, nrhs, (const __nv_bfloat162*)inv, r, x, g_sel.list);
+    launch_pdl(grid, 32 * wpb, 0, s, k_dense_apply_lp<__nv_bfloat162>, N, nrhs, (const __nv_bfloat162*)inv, r, x, g_sel.list);
   else
-    k_dense_apply_lp<float2><<<grid, 32 * wpb, 0, s>>>(N, nrhs, (const float2*)inv, r, x, g_sel.list);
+    launch_pdl(grid, 32 * wpb, 0, s, k_dense_apply_lp<float2>, N, nrhs, (const float2*)inv, r, x, g_sel.list);
 }
 
 template void launch_dense_apply<float>(int, int, int, const double2*, const float2*, float2*, cudaStream_t);

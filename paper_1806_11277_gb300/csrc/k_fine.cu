@@ -30,7 +30,7 @@ __device__ __forceinline__ Coef4<T> ldcf(const Coef4<T>* p, long long c) {
   }
   return r;
 }
-template <typename C> __device__ __forceinline__ C ldc(const C* p, long long i) { return __ldg(p + i); }
+template <typename C> __device__ __forceinline__ C ldc(const C* p, long long i) { return p[i]; }
 
 template <typename T> struct FineP {
   T h2inv, hinv, alpha;
@@ -92,9 +92,10 @@ __device__ __forceinline__ typename CT<T>::type row_p(
 
 template <typename T, int D>
 __global__ void k_fine_apply(Grid g, int nrhs, const Coef4<T>* __restrict__ cf, FineP<T> P,
-                             const typename CT<T>::type* __restrict__ x,
-                             const typename CT<T>::type* __restrict__ b,
-                             typename CT<T>::type* __restrict__ y, int mode, const int* __restrict__ il) {
+                             const typename CT<T>::type* x,
+                             const typename CT<T>::type* b,
+                             typename CT<T>::type* __restrict__ y, int mode, const int* il) {
+  pdl_enter();
   typedef typename CT<T>::type C;
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
@@ -133,9 +134,10 @@ __global__ void k_fine_apply(Grid g, int nrhs, const Coef4<T>* __restrict__ cf, 
 // is solved in closed form through the pressure Schur complement.
 template <typename T, int D, bool FULL>
 __global__ void k_fine_vanka(Grid g, int nrhs, const Coef4<T>* __restrict__ cf, FineP<T> P,
-                             T wu, T wp, int colour, const typename CT<T>::type* __restrict__ b,
-                             const typename CT<T>::type* __restrict__ xi,
-                             typename CT<T>::type* __restrict__ xo, const int* __restrict__ il) {
+                             T wu, T wp, int colour, const typename CT<T>::type* b,
+                             const typename CT<T>::type* xi,
+                             typename CT<T>::type* __restrict__ xo, const int* il) {
+  pdl_enter();
   typedef typename CT<T>::type C;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long npair = g.ncell >> 1;
@@ -279,9 +281,10 @@ __device__ __forceinline__ void cp_async_wait_all() {
 
 __global__ void __launch_bounds__(VT_X * VT_Y / 2) k_fine_vanka_tile(Grid g, int nrhs, const Coef4<float>* __restrict__ cf,
                                                                      FineP<float> P, float wu, float wp, int colour,
-                                                                     const float2* __restrict__ b,
-                                                                     const float2* __restrict__ xi,
-                                                                     float2* __restrict__ xo, const int* __restrict__ il) {
+                                                                     const float2* b,
+                                                                     const float2* xi,
+                                                                     float2* __restrict__ xo, const int* il) {
+  pdl_enter();
   __shared__ __align__(16) float2 xs[3][VS_Y][VS_X];
   __shared__ __align__(16) float4 cs[VS_Y][VS_X];
   const int item = il ? il[blockIdx.z] : blockIdx.z;
@@ -344,11 +347,11 @@ __global__ void __launch_bounds__(VT_X * VT_Y / 2) k_fine_vanka_tile(Grid g, int
   for (int k = 0; k < 2; ++k) {
     const long long sk = k == 0 ? 1 : nx;
     ok[k] = ic[k] >= 1;
-    if (ok[k]) r[k] = csub(__ldg(bb + (long long)k * N + c), row_u(k, sx, sy, &dg[k]));
+    if (ok[k]) r[k] = csub(*(bb + (long long)k * N + c), row_u(k, sx, sy, &dg[k]));
     else { r[k] = make_float2(0.f, 0.f); dg[k] = make_float2(1.f, 0.f); }
     g_[k] = make_float2(P.hinv, 0.f);
     ok[2 + k] = ic[k] + 1 < nn[k];
-    if (ok[2 + k]) r[2 + k] = csub(__ldg(bb + (long long)k * N + c + sk), row_u(k, sx + (k == 0), sy + (k == 1), &dg[2 + k]));
+    if (ok[2 + k]) r[2 + k] = csub(*(bb + (long long)k * N + c + sk), row_u(k, sx + (k == 0), sy + (k == 1), &dg[2 + k]));
     else { r[2 + k] = make_float2(0.f, 0.f); dg[2 + k] = make_float2(1.f, 0.f); }
     g_[2 + k] = make_float2(-P.hinv, 0.f);
   }
@@ -359,7 +362,7 @@ __global__ void __launch_bounds__(VT_X * VT_Y / 2) k_fine_vanka_tile(Grid g, int
     sdiv = csub(sdiv, xs[0][sy][sx + 1]);
     sdiv = cadd(sdiv, xs[1][sy][sx]);
     sdiv = csub(sdiv, xs[1][sy + 1][sx]);
-    r[4] = csub(__ldg(bb + 2 * N + c), cadd(y, cscale(sdiv, P.hinv)));
+    r[4] = csub(*(bb + 2 * N + c), cadd(y, cscale(sdiv, P.hinv)));
   }
   float2 sch = make_float2(-cc.y, 0.f);
   float2 rp = r[4];
@@ -553,8 +556,8 @@ void launch_fine_apply(const Grid& g, int items, int nrhs, const Coef4<float>* c
   const FineP<float> P = mkP<float>(h, alpha);
   const int bs = spread_bs(g.ncell, items, 256);
   const dim3 gr((unsigned)((g.ncell + bs - 1) / bs), sel_items(items));
-  if (g.d == 2) k_fine_apply<float, 2><<<gr, bs, 0, s>>>(g, nrhs, cf, P, x, b, y, mode, g_sel.list);
-  else k_fine_apply<float, 3><<<gr, bs, 0, s>>>(g, nrhs, cf, P, x, b, y, mode, g_sel.list);
+  if (g.d == 2) launch_pdl(gr, bs, 0, s, k_fine_apply<float, 2>, g, nrhs, cf, P, x, b, y, mode, g_sel.list);
+  else launch_pdl(gr, bs, 0, s, k_fine_apply<float, 3>, g, nrhs, cf, P, x, b, y, mode, g_sel.list);
 }
 
 template <typename T>
@@ -566,7 +569,7 @@ void launch_fine_vanka(const Grid& g, int items, int nrhs, const Coef4<T>* cf, d
   if constexpr (sizeof(T) == 4) {
     if (g.d == 2 && !full && g.n[0] % VT_X == 0 && g.n[1] % VT_Y == 0) {   // shared-memory tiles
       const dim3 gt(g.n[0] / VT_X, g.n[1] / VT_Y, sel_items(items));
-      k_fine_vanka_tile<<<gt, VT_X * VT_Y / 2, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+      launch_pdl(gt, VT_X * VT_Y / 2, 0, s, k_fine_vanka_tile, g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
       return;
     }
   }
@@ -574,11 +577,11 @@ void launch_fine_vanka(const Grid& g, int items, int nrhs, const Coef4<T>* cf, d
   const int bs = spread_bs(np, items, 128);
   const dim3 gr((unsigned)((np + bs - 1) / bs), sel_items(items));
   if (g.d == 2) {
-    if (full) k_fine_vanka<T, 2, true><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
-    else k_fine_vanka<T, 2, false><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    if (full) launch_pdl(gr, bs, 0, s, k_fine_vanka<T, 2, true>, g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    else launch_pdl(gr, bs, 0, s, k_fine_vanka<T, 2, false>, g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
   } else {
-    if (full) k_fine_vanka<T, 3, true><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
-    else k_fine_vanka<T, 3, false><<<gr, bs, 0, s>>>(g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    if (full) launch_pdl(gr, bs, 0, s, k_fine_vanka<T, 3, true>, g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
+    else launch_pdl(gr, bs, 0, s, k_fine_vanka<T, 3, false>, g, nrhs, cf, P, wu, wp, colour, b, xi, xo, g_sel.list);
   }
 }
 

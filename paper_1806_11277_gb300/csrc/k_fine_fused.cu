@@ -99,7 +99,7 @@ __device__ __forceinline__ void cpa_wait() {
 }
 
 // (P e_c) of component a at fine cell (gx, gy): coarse item vector ec ([3][ncc])
-__device__ __forceinline__ float2 prolong_at(const float2* __restrict__ ec, int a, int gx, int gy, int ncx,
+__device__ __forceinline__ float2 prolong_at(const float2* ec, int a, int gx, int gy, int ncx,
                                              int ncy) {
   const int kx = a == 2 ? 2 : (a == 0 ? 0 : 1);
   const int ky = a == 2 ? 2 : (a == 1 ? 0 : 1);
@@ -111,13 +111,13 @@ __device__ __forceinline__ float2 prolong_at(const float2* __restrict__ ec, int 
   float2 acc = make_float2(0.f, 0.f);
   if (wy0 != 0.0f) {
     const float2* row = e + (long long)Y0 * ncx;
-    if (wx0 != 0.0f) acc = cfma(make_float2(wy0 * wx0, 0.f), __ldg(row + X0), acc);
-    if (wx1 != 0.0f) acc = cfma(make_float2(wy0 * wx1, 0.f), __ldg(row + X1), acc);
+    if (wx0 != 0.0f) acc = cfma(make_float2(wy0 * wx0, 0.f), *(row + X0), acc);
+    if (wx1 != 0.0f) acc = cfma(make_float2(wy0 * wx1, 0.f), *(row + X1), acc);
   }
   if (wy1 != 0.0f) {
     const float2* row = e + (long long)Y1 * ncx;
-    if (wx0 != 0.0f) acc = cfma(make_float2(wy1 * wx0, 0.f), __ldg(row + X0), acc);
-    if (wx1 != 0.0f) acc = cfma(make_float2(wy1 * wx1, 0.f), __ldg(row + X1), acc);
+    if (wx0 != 0.0f) acc = cfma(make_float2(wy1 * wx0, 0.f), *(row + X0), acc);
+    if (wx1 != 0.0f) acc = cfma(make_float2(wy1 * wx1, 0.f), *(row + X1), acc);
   }
   return acc;
 }
@@ -195,24 +195,40 @@ __global__ void k_sweep_tables_schur(Grid g, const float4* __restrict__ cf, FP P
   sinv[c] = cinv(make_float2(-kap - P.h2inv * sd.x, -P.h2inv * sd.y));
 }
 
-// Stage the tile (x0, y0) of x: from xv (null: the zero iterate), plus P e when e is
-// given, zero outside the grid and on Dirichlet slots; with mu / h^2 and
-// 1/(lambda+mu) of the (clamped) cells and the setup-time tables: fx, fy the
-// face diagonals or their inverses (tx, ty), mm the inverse Schur complements (ts;
-// not staged when null), vm the vertex means (tv).
+// Stage the coefficients of the tile (x0, y0): mu / h^2 and 1/(lambda+mu) of the (clamped) cells and the setup-time
+// tables: fx, fy the face diagonals or their inverses (tx, ty), mm the inverse Schur complements (ts; not staged
+// when null), vm the vertex means (tv).  Setup-time data only: runs before the kernel waits for the launch
+// before it (launch_pdl).
 template <int W, int H, int NT>
 __device__ __forceinline__ void stage_tab(Tile<W, H>& S, const float4* __restrict__ cfs, const float2* __restrict__ tx,
                                           const float2* __restrict__ ty, const float2* __restrict__ ts,
-                                          const float* __restrict__ tv, const float2* __restrict__ xv,
-                                          const float2* __restrict__ e, const Grid& gc, int N, int nx, int ny,
-                                          int x0, int y0, float h2inv) {
+                                          const float* __restrict__ tv, int nx, int ny, int x0, int y0, float h2inv) {
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < W * H; idx += NT) {
+    const int lx = idx % W, ly = idx / W;
+    const int gx = x0 + lx, gy = y0 + ly;
+    const int gcl = min(max(gy, 0), ny - 1) * nx + min(max(gx, 0), nx - 1);   // a valid address in every case
+    cpa8(&S.fx[ly][lx], tx + gcl, 8);
+    cpa8(&S.fy[ly][lx], ty + gcl, 8);
+    if (ts) cpa8(&S.mm[ly][lx], ts + gcl, 8);
+    cpa4(&S.vm[ly][lx], tv + min(max(gy, 0), ny) * (nx + 1) + min(max(gx, 0), nx));
+    const float2 mk = __ldg(reinterpret_cast<const float2*>(cfs + gcl));   // mu, 1/(lambda+mu)
+    S.mu[ly][lx] = mk.x * h2inv;
+    S.kap[ly][lx] = mk.y;
+  }
+}
+
+// Stage x of the tile: from xv (null: the zero iterate), plus P e when e is given, zero outside the grid and on
+// Dirichlet slots.
+template <int W, int H, int NT>
+__device__ __forceinline__ void stage_x(Tile<W, H>& S, const float2* xv, const float2* e, const Grid& gc, int N, int nx,
+                                        int ny, int x0, int y0) {
 #pragma unroll 4
   for (int idx = threadIdx.x; idx < W * H; idx += NT) {
     const int lx = idx % W, ly = idx / W;
     const int gx = x0 + lx, gy = y0 + ly;
     const bool in = gx >= 0 && gx < nx && gy >= 0 && gy < ny;
-    const int cx = min(max(gx, 0), nx - 1), cy = min(max(gy, 0), ny - 1);
-    const int gcl = cy * nx + cx;                                  // a valid address in every case
+    const int gcl = min(max(gy, 0), ny - 1) * nx + min(max(gx, 0), nx - 1);
     const bool v0 = in && gx >= 1, v1 = in && gy >= 1;            // u_k slot 0 is a boundary face
     if (!e) {
       if (xv) {
@@ -225,18 +241,11 @@ __device__ __forceinline__ void stage_tab(Tile<W, H>& S, const float4* __restric
       }
     } else {
       float2 u0 = make_float2(0.f, 0.f), u1 = u0, pv = u0;
-      if (v0) u0 = cadd(xv ? __ldg(xv + gcl) : u0, prolong_at(e, 0, gx, gy, gc.n[0], gc.n[1]));
-      if (v1) u1 = cadd(xv ? __ldg(xv + N + gcl) : u1, prolong_at(e, 1, gx, gy, gc.n[0], gc.n[1]));
-      if (in) pv = cadd(xv ? __ldg(xv + 2 * N + gcl) : pv, prolong_at(e, 2, gx, gy, gc.n[0], gc.n[1]));
+      if (v0) u0 = cadd(xv ? xv[gcl] : u0, prolong_at(e, 0, gx, gy, gc.n[0], gc.n[1]));
+      if (v1) u1 = cadd(xv ? xv[N + gcl] : u1, prolong_at(e, 1, gx, gy, gc.n[0], gc.n[1]));
+      if (in) pv = cadd(xv ? xv[2 * N + gcl] : pv, prolong_at(e, 2, gx, gy, gc.n[0], gc.n[1]));
       S.x[0][ly][lx] = u0; S.x[1][ly][lx] = u1; S.x[2][ly][lx] = pv;
     }
-    cpa8(&S.fx[ly][lx], tx + gcl, 8);
-    cpa8(&S.fy[ly][lx], ty + gcl, 8);
-    if (ts) cpa8(&S.mm[ly][lx], ts + gcl, 8);
-    cpa4(&S.vm[ly][lx], tv + min(max(gy, 0), ny) * (nx + 1) + min(max(gx, 0), nx));
-    const float2 mk = __ldg(reinterpret_cast<const float2*>(cfs + gcl));   // mu, 1/(lambda+mu)
-    S.mu[ly][lx] = mk.x * h2inv;
-    S.kap[ly][lx] = mk.y;
   }
 }
 
@@ -273,7 +282,7 @@ __device__ __forceinline__ float2 face_rhs(float2 b, float wpn, float2 xnp, floa
 // S = -kap - sum_a g_a^2 / dg_a (stored inverted per cell).
 template <int W, int H>
 __device__ __forceinline__ void cell_update(const Tile<W, H>& S, int sx, int sy, int gx, int gy, int nx, int ny,
-                                            int N, int c, const float2* __restrict__ bb, const FP& P,
+                                            int N, int c, const float2* bb, const FP& P,
                                             float wu, float wp, float2 o[5], bool ok[4]) {
   ok[0] = gx >= 1;
   ok[1] = gy >= 1;
@@ -281,9 +290,9 @@ __device__ __forceinline__ void cell_update(const Tile<W, H>& S, int sx, int sy,
   ok[3] = gy + 1 < ny;
   // right-hand sides first (global loads in flight while the rows are formed)
   const float2 z = make_float2(0.f, 0.f);
-  const float2 b0 = ok[0] ? __ldg(bb + c) : z, b1 = ok[1] ? __ldg(bb + N + c) : z;
-  const float2 b2 = ok[2] ? __ldg(bb + c + 1) : z, b3 = ok[3] ? __ldg(bb + N + c + nx) : z;
-  const float2 b4 = __ldg(bb + 2 * N + c);
+  const float2 b0 = ok[0] ? *(bb + c) : z, b1 = ok[1] ? *(bb + N + c) : z;
+  const float2 b2 = ok[2] ? *(bb + c + 1) : z, b3 = ok[3] ? *(bb + N + c + nx) : z;
+  const float2 b4 = *(bb + 2 * N + c);
   // every staged value the five rows read, once
   const float2 u0m = S.x[0][sy][sx - 1], u00 = S.x[0][sy][sx], u01 = S.x[0][sy][sx + 1], u02 = S.x[0][sy][sx + 2];
   const float2 u0dn = S.x[0][sy - 1][sx], u0up = S.x[0][sy + 1][sx];
@@ -339,10 +348,11 @@ __global__ void __launch_bounds__(SW_T, 4) k_fine_sweep_tile(Grid g, Grid gc, in
                                                              const float2* __restrict__ tsi,
                                                              const float* __restrict__ tvm,
                                                              FP P, float wu, float wp,
-                                                             const float2* __restrict__ b,
-                                                             const float2* __restrict__ xi,
-                                                             const float2* __restrict__ ec,
-                                                             float2* __restrict__ xo, const int* __restrict__ il) {
+                                                             const float2* b,
+                                                             const float2* xi,
+                                                             const float2* ec,
+                                                             float2* __restrict__ xo, const int* il) {
+  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SweepTile& S = *reinterpret_cast<SweepTile*>(smem_raw);
   const int item = il ? il[blockIdx.z] : blockIdx.z;
@@ -357,7 +367,9 @@ __global__ void __launch_bounds__(SW_T, 4) k_fine_sweep_tile(Grid g, Grid gc, in
   const int set = item / nrhs;
   const long long nvt = (long long)(nx + 1) * (ny + 1);
   stage_tab<SWS_X, SWS_Y, SW_T>(S, cfs, tdx + (long long)set * N, tdy + (long long)set * N, tsi + (long long)set * N,
-                                tvm + set * nvt, x, e, gc, N, nx, ny, x0, y0, P.h2inv);
+                                tvm + set * nvt, nx, ny, x0, y0, P.h2inv);
+  pdl_wait();
+  stage_x<SWS_X, SWS_Y, SW_T>(S, x, e, gc, N, nx, ny, x0, y0);
   cpa_wait();
   __syncthreads();
   const float2* bb = b + vo;
@@ -422,10 +434,11 @@ __global__ void __launch_bounds__(RR_T, 4) k_fine_resid_restrict_tile(Grid g, Gr
                                                                       const float2* __restrict__ tgx,
                                                                       const float2* __restrict__ tgy,
                                                                       const float* __restrict__ tvm, FP P,
-                                                                      const float2* __restrict__ x,
-                                                                      const float2* __restrict__ b,
+                                                                      const float2* x,
+                                                                      const float2* b,
                                                                       float2* __restrict__ rc,
-                                                                      const int* __restrict__ il) {
+                                                                      const int* il) {
+  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ResTile& S = *reinterpret_cast<ResTile*>(smem_raw);
   const int item = il ? il[blockIdx.z] : blockIdx.z;
@@ -437,8 +450,10 @@ __global__ void __launch_bounds__(RR_T, 4) k_fine_resid_restrict_tile(Grid g, Gr
   const int x0 = X0 - RR_H, y0 = Y0 - RR_H;
   const int set = item / nrhs;
   const long long nvt = (long long)(nx + 1) * (ny + 1);
-  stage_tab<RRS_X, RRS_Y, RR_T>(S, cfs, tgx + (long long)set * N, tgy + (long long)set * N, nullptr, tvm + set * nvt,
-                                x + vo, nullptr, gc, N, nx, ny, x0, y0, P.h2inv);
+  stage_tab<RRS_X, RRS_Y, RR_T>(S, cfs, tgx + (long long)set * N, tgy + (long long)set * N, nullptr, tvm + set * nvt, nx,
+                                ny, x0, y0, P.h2inv);
+  pdl_wait();
+  stage_x<RRS_X, RRS_Y, RR_T>(S, x + vo, nullptr, gc, N, nx, ny, x0, y0);
   cpa_wait();
   __syncthreads();
   const float2* bb = b + vo;
@@ -457,9 +472,9 @@ __global__ void __launch_bounds__(RR_T, 4) k_fine_resid_restrict_tile(Grid g, Gr
     const int sx = gx - x0, sy = gy - y0;
     const int c = gy * nx + gx;
     const float2 z = make_float2(0.f, 0.f);
-    const float2 b0 = gx >= 1 ? __ldg(bb + c) : z;
-    const float2 b1 = gy >= 1 ? __ldg(bb + N + c) : z;
-    const float2 b2 = __ldg(bb + 2 * N + c);
+    const float2 b0 = gx >= 1 ? *(bb + c) : z;
+    const float2 b1 = gy >= 1 ? *(bb + N + c) : z;
+    const float2 b2 = *(bb + 2 * N + c);
     const float2 u0m = S.x[0][sy][sx - 1], u00 = S.x[0][sy][sx], u01 = S.x[0][sy][sx + 1];
     const float2 u0dn = S.x[0][sy - 1][sx], u0up = S.x[0][sy + 1][sx];
     const float2 v0m = S.x[1][sy - 1][sx], v00 = S.x[1][sy][sx], v01 = S.x[1][sy + 1][sx];
@@ -566,7 +581,7 @@ void launch_fine_sweep_tile(const Grid& g, const Grid& gc, int items, int nrhs, 
   const FP P = make_fp(h, alpha);
   smem_attr(k_fine_sweep_tile, sizeof(SweepTile));
   const dim3 gr(g.n[0] / SW_X, g.n[1] / SW_Y, sel_items(items));
-  k_fine_sweep_tile<<<gr, SW_T, sizeof(SweepTile), s>>>(g, gc, nrhs, reinterpret_cast<const float4*>(cf), T.dvx,
+  launch_pdl(gr, SW_T, sizeof(SweepTile), s, k_fine_sweep_tile, g, gc, nrhs, reinterpret_cast<const float4*>(cf), T.dvx,
                                                          T.dvy, T.sinv, T.vm, P, wu, wp, b, xi, ec, xo, g_sel.list);
 }
 
@@ -576,7 +591,7 @@ void launch_fine_resid_restrict_tile(const Grid& g, const Grid& gc, int items, i
   const FP P = make_fp(h, alpha);
   smem_attr(k_fine_resid_restrict_tile, sizeof(ResTile));
   const dim3 gr(g.n[0] / RR_X, g.n[1] / RR_Y, sel_items(items));
-  k_fine_resid_restrict_tile<<<gr, RR_T, sizeof(ResTile), s>>>(g, gc, nrhs, reinterpret_cast<const float4*>(cf),
+  launch_pdl(gr, RR_T, sizeof(ResTile), s, k_fine_resid_restrict_tile, g, gc, nrhs, reinterpret_cast<const float4*>(cf),
                                                                 T.gdx, T.gdy, T.vm, P, x, b, rc, g_sel.list);
 }
 

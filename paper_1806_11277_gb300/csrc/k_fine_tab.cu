@@ -117,93 +117,127 @@ __global__ void k_fine_tab_schur(Grid g, const Coef4<double>* __restrict__ cf, d
   F.sinv[o] = mk<T>((T)v.x, (T)v.y);
 }
 
-// off-diagonal part of the u_k row at face (cell) c with coordinates i, added to s with a minus sign of the
-// operator's: s + sum of weights * neighbours - (p_c - p_{c - e_k}) / h
+// weights of the u_k row's neighbours at face (cell) c with coordinates i (zero towards what is no unknown)
+template <typename T, int D> struct RowW {
+  T p, m, tp[D], tm[D];
+};
 template <typename T, int D>
-__device__ __forceinline__ typename CT<T>::type off_row(const Grid& g, int k, int c, const int i[3], const FineTab<T>& F,
-                                                        long long so, const typename CT<T>::type* __restrict__ x,
-                                                        long long N, T hinv, typename CT<T>::type s) {
+__device__ __forceinline__ RowW<T, D> row_weights(const Grid& g, int k, int c, const int i[3], const FineTab<T>& F,
+                                                  long long so) {
+  RowW<T, D> w;
+  const T* mu = F.muh + so;
+  w.p = i[k] + 1 < g.n[k] ? __ldg(mu + c) : T(0);
+  w.m = __ldg(mu + c - (int)stride_of(g, k));
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    w.tp[j] = w.tm[j] = 0;
+    if (j == k) continue;
+    const T* em = F.em[k < j ? pair_of(k, j) : pair_of(j, k)] + so;
+    if (i[j] + 1 < g.n[j]) w.tp[j] = __ldg(em + c + (int)stride_of(g, j));
+    if (i[j] >= 1) w.tm[j] = __ldg(em + c);
+  }
+  return w;
+}
+// s + sum of weights * neighbours - (p_c - p_{c - e_k}) / h: minus the row's off-diagonal part
+template <typename T, int D>
+__device__ __forceinline__ typename CT<T>::type off_row(const Grid& g, int k, int c, const int i[3],
+                                                        const RowW<T, D>& w, const typename CT<T>::type* x, long long N,
+                                                        T hinv, typename CT<T>::type s) {
   typedef typename CT<T>::type C;
   const int sk = (int)stride_of(g, k);
   const C* xk = x + (long long)k * N;
   const C* p = x + (long long)D * N;
-  const T* mu = F.muh + so;
-  C xp = czero<C>(), xm = czero<C>();
-  T wp = 0;
-  const T wm = __ldg(mu + c - sk);
-  if (i[k] + 1 < g.n[k]) { xp = __ldg(xk + c + sk); wp = __ldg(mu + c); }
-  if (i[k] - 1 >= 1) xm = __ldg(xk + c - sk);
-  const C pc = __ldg(p + c), pm = __ldg(p + c - sk);
-  C tp[D], tm[D];
-  T vp[D], vm[D];
+  C xp = czero<C>(), xm = czero<C>(), tp[D], tm[D];
+  if (i[k] + 1 < g.n[k]) xp = xk[c + sk];
+  if (i[k] - 1 >= 1) xm = xk[c - sk];
+  const C pc = p[c], pm = p[c - sk];
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     tp[j] = tm[j] = czero<C>();
-    vp[j] = vm[j] = 0;
     if (j == k) continue;
     const int sj = (int)stride_of(g, j);
-    const T* em = F.em[k < j ? pair_of(k, j) : pair_of(j, k)] + so;
-    if (i[j] + 1 < g.n[j]) { tp[j] = __ldg(xk + c + sj); vp[j] = __ldg(em + c + sj); }
-    if (i[j] >= 1) { tm[j] = __ldg(xk + c - sj); vm[j] = __ldg(em + c); }
+    if (i[j] + 1 < g.n[j]) tp[j] = xk[c + sj];
+    if (i[j] >= 1) tm[j] = xk[c - sj];
   }
-  s = rfma(wp, xp, s);
-  s = rfma(wm, xm, s);
+  s = rfma(w.p, xp, s);
+  s = rfma(w.m, xm, s);
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     if (j == k) continue;
-    s = rfma(vp[j], tp[j], s);
-    s = rfma(vm[j], tm[j], s);
+    s = rfma(w.tp[j], tp[j], s);
+    s = rfma(w.tm[j], tm[j], s);
   }
   return rfma(-hinv, csub(pc, pm), s);
 }
 
 // Thread = pair of cells along x; the cell of the colour is relaxed, the other one's pressure copied (as k_fine_vanka).
 // With t_a = (b_a - offdiag_a) / dg_a - x_a: dp = (r_p - sum_a g_a t_a) / S, du_a = t_a - g_a dp / dg_a,
-// g = +1/h on the low faces, -1/h on the high ones.
+// g = +1/h on the low faces, -1/h on the high ones.  Everything the tables hold is loaded before the wait for the
+// launch before (launch_pdl).
 template <typename T, int D>
 __global__ void k_fine_vanka_tab(Grid g, int nrhs, FineTab<T> F, T hinv, T wu, T wp, int colour,
-                                 const typename CT<T>::type* __restrict__ b, const typename CT<T>::type* __restrict__ xi,
-                                 typename CT<T>::type* __restrict__ xo, const int* __restrict__ il) {
+                                 const typename CT<T>::type* b, const typename CT<T>::type* xi,
+                                 typename CT<T>::type* __restrict__ xo, const int* il) {
+  pdl_trigger();
   typedef typename CT<T>::type C;
   const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long N = g.ncell;
-  if (t0 >= N / 2) return;
-  const int item = il ? il[blockIdx.y] : blockIdx.y;
+  const bool live = t0 < N / 2;
+  const int item = il ? il[blockIdx.y] : blockIdx.y;   // not changed while a cycle runs
   const long long vo = (long long)item * (D + 1) * N, so = (long long)(item / nrhs) * N;
+  int c = (int)(2 * t0);
+  int i[3] = {0, 0, 0};
+  RowW<T, D> w[2 * D];
+  C dv[2 * D], sinv = czero<C>();
+  T kap = 0;
+  bool ok[2 * D];
+  if (live) {
+    cell_coords(g, c, i);
+    if (((i[0] + i[1] + i[2]) & 1) != colour) { ++c; ++i[0]; }
+#pragma unroll
+    for (int a = 0; a < 2 * D; ++a) {
+      const int k = a % D, hi = a >= D, cc = c + (hi ? (int)stride_of(g, k) : 0);
+      int ia[3] = {i[0], i[1], i[2]};
+      ia[k] += hi;
+      ok[a] = ia[k] >= 1 && ia[k] < g.n[k];
+      dv[a] = czero<C>();
+      if (ok[a]) {
+        dv[a] = __ldg(F.dv[k] + so + cc);
+        w[a] = row_weights<T, D>(g, k, cc, ia, F, so);
+      }
+    }
+    kap = __ldg(F.kap + so + c);
+    sinv = __ldg(F.sinv + so + c);
+  }
+  pdl_wait();
+  if (!live) return;
   const C* x = xi + vo;
   const C* bb = b + vo;
   C* xout = xo + vo;
-  int c = (int)(2 * t0);
-  int i[3];
-  cell_coords(g, c, i);
-  if (((i[0] + i[1] + i[2]) & 1) != colour) { ++c; ++i[0]; }
   const int co = (c & 1) ? c - 1 : c + 1;
-  xout[(long long)D * N + co] = __ldg(x + (long long)D * N + co);
-  const C pc = __ldg(x + (long long)D * N + c);
-  C t[2 * D], xv[2 * D], dv[2 * D];
-  bool ok[2 * D];
+  xout[(long long)D * N + co] = x[(long long)D * N + co];
+  const C pc = x[(long long)D * N + c];
+  C t[2 * D], xv[2 * D];
   C dsum = czero<C>();                              // sum over the faces of (low - high) x
 #pragma unroll
   for (int a = 0; a < 2 * D; ++a) {
     const int k = a % D, hi = a >= D, cc = c + (hi ? (int)stride_of(g, k) : 0);
     int ia[3] = {i[0], i[1], i[2]};
     ia[k] += hi;
-    ok[a] = ia[k] >= 1 && ia[k] < g.n[k];
-    t[a] = xv[a] = dv[a] = czero<C>();
+    t[a] = xv[a] = czero<C>();
     if (ok[a]) {
-      xv[a] = __ldg(x + (long long)k * N + cc);
-      dv[a] = __ldg(F.dv[k] + so + cc);
-      const C s = off_row<T, D>(g, k, cc, ia, F, so, x, N, hinv, __ldg(bb + (long long)k * N + cc));
+      xv[a] = x[(long long)k * N + cc];
+      const C s = off_row<T, D>(g, k, cc, ia, w[a], x, N, hinv, bb[(long long)k * N + cc]);
       t[a] = csub(cmulf<T>(dv[a], s), xv[a]);
     }
     dsum = hi ? csub(dsum, xv[a]) : cadd(dsum, xv[a]);
   }
   // pressure row residual and the block's Schur complement; t is zero on faces that are not unknowns
-  C rp = __ldg(bb + (long long)D * N + c);
-  rp = rfma(__ldg(F.kap + so + c), pc, rfma(-hinv, dsum, rp));
+  C rp = bb[(long long)D * N + c];
+  rp = rfma(kap, pc, rfma(-hinv, dsum, rp));
 #pragma unroll
   for (int a = 0; a < 2 * D; ++a) rp = rfma(a >= D ? hinv : -hinv, t[a], rp);
-  const C dp = cmulf<T>(rp, __ldg(F.sinv + so + c));
+  const C dp = cmulf<T>(rp, sinv);
   xout[(long long)D * N + c] = rfma(wp, dp, pc);
 #pragma unroll
   for (int a = 0; a < 2 * D; ++a) {
@@ -217,8 +251,9 @@ __global__ void k_fine_vanka_tab(Grid g, int nrhs, FineTab<T> F, T hinv, T wu, T
 // y = K x (mode 0) or b - K x (mode 1), alpha = shift
 template <typename T, int D>
 __global__ void k_fine_apply_tab(Grid g, int nrhs, FineTab<T> F, T hinv, T alpha,
-                                 const typename CT<T>::type* __restrict__ xi, const typename CT<T>::type* __restrict__ b,
-                                 typename CT<T>::type* __restrict__ y, int mode, const int* __restrict__ il) {
+                                 const typename CT<T>::type* xi, const typename CT<T>::type* b,
+                                 typename CT<T>::type* __restrict__ y, int mode, const int* il) {
+  pdl_enter();
   typedef typename CT<T>::type C;
   const long long c0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long N = g.ncell;
@@ -234,21 +269,21 @@ __global__ void k_fine_apply_tab(Grid g, int nrhs, FineTab<T> F, T hinv, T alpha
     const long long o = (long long)k * N + c;
     C r = czero<C>();
     if (i[k] >= 1) {
-      const C xc = __ldg(x + o);
+      const C xc = *(x + o);
       C dg = __ldg(F.dg[k] + so + c);
       dg.y = fma(alpha, __ldg(F.rf[k] + so + c), dg.y);
       dsum = cadd(dsum, xc);
-      const C off = off_row<T, D>(g, k, c, i, F, so, x, N, hinv, mode ? __ldg(b + vo + o) : czero<C>());
+      const C off = off_row<T, D>(g, k, c, i, row_weights<T, D>(g, k, c, i, F, so), x, N, hinv, mode ? *(b + vo + o) : czero<C>());
       const C dx = cmulf<T>(dg, xc);
       r = mode ? csub(off, dx) : csub(dx, off);
     }
-    if (i[k] + 1 < g.n[k]) dsum = csub(dsum, __ldg(x + o + stride_of(g, k)));
+    if (i[k] + 1 < g.n[k]) dsum = csub(dsum, *(x + o + stride_of(g, k)));
     y[vo + o] = r;
   }
   const long long o = (long long)D * N + c;
-  C r = rfma(-__ldg(F.kap + so + c), __ldg(x + o), czero<C>());
+  C r = rfma(-__ldg(F.kap + so + c), *(x + o), czero<C>());
   r = rfma(hinv, dsum, r);
-  if (mode) r = csub(__ldg(b + vo + o), r);
+  if (mode) r = csub(*(b + vo + o), r);
   y[vo + o] = r;
 }
 
@@ -275,8 +310,8 @@ void launch_fine_vanka_tab(const Grid& g, int items, int nrhs, const FineTab<T>&
   const int bs = spread_bs(g.ncell / 2, items, 128);
   const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs), sel_items(items));
   const T hinv = (T)(1.0 / h);
-  if (g.d == 2) k_fine_vanka_tab<T, 2><<<gr, bs, 0, s>>>(g, nrhs, F, hinv, wu, wp, colour, b, xi, xo, g_sel.list);
-  else k_fine_vanka_tab<T, 3><<<gr, bs, 0, s>>>(g, nrhs, F, hinv, wu, wp, colour, b, xi, xo, g_sel.list);
+  if (g.d == 2) launch_pdl(gr, bs, 0, s, k_fine_vanka_tab<T, 2>, g, nrhs, F, hinv, wu, wp, colour, b, xi, xo, g_sel.list);
+  else launch_pdl(gr, bs, 0, s, k_fine_vanka_tab<T, 3>, g, nrhs, F, hinv, wu, wp, colour, b, xi, xo, g_sel.list);
 }
 
 void launch_fine_apply_tab(const Grid& g, int items, int nrhs, const FineTab<double>& F, double h, double alpha,
@@ -284,8 +319,8 @@ void launch_fine_apply_tab(const Grid& g, int items, int nrhs, const FineTab<dou
   const int bs = spread_bs(g.ncell, items, 128);
   const dim3 gr((unsigned)((g.ncell + bs - 1) / bs), sel_items(items));
   const double hinv = 1.0 / h;
-  if (g.d == 2) k_fine_apply_tab<double, 2><<<gr, bs, 0, s>>>(g, nrhs, F, hinv, alpha, x, b, y, mode, g_sel.list);
-  else k_fine_apply_tab<double, 3><<<gr, bs, 0, s>>>(g, nrhs, F, hinv, alpha, x, b, y, mode, g_sel.list);
+  if (g.d == 2) launch_pdl(gr, bs, 0, s, k_fine_apply_tab<double, 2>, g, nrhs, F, hinv, alpha, x, b, y, mode, g_sel.list);
+  else launch_pdl(gr, bs, 0, s, k_fine_apply_tab<double, 3>, g, nrhs, F, hinv, alpha, x, b, y, mode, g_sel.list);
 }
 
 #define INST(T)                                                                                                       \

@@ -39,18 +39,19 @@ __device__ __forceinline__ void block_store(double2* acc, int nv, double2* part,
   }
 }
 
-__global__ void k_mdot(long long n, int items, int nv, const double2* __restrict__ V,
-                       const double2* __restrict__ w, double2* part, int nblk) {
+__global__ void k_mdot(long long n, int items, int nv, const double2* V,
+                       const double2* w, double2* part, int nblk) {
+  pdl_enter();
   const int item = blockIdx.y;
   double2 acc[MAXV];
   for (int i = 0; i < MAXV; ++i) acc[i] = make_double2(0, 0);
   const double2* wv = w + (long long)item * n;
   for (long long e = (long long)blockIdx.x * KB + threadIdx.x; e < n; e += (long long)nblk * KB) {
-    const double2 we = __ldg(wv + e);
+    const double2 we = *(wv + e);
 #pragma unroll
     for (int i = 0; i < MAXV; ++i) {
       if (i < nv) {
-        const double2 v = __ldg(V + ((long long)i * items + item) * n + e);
+        const double2 v = *(V + ((long long)i * items + item) * n + e);
         acc[i].x = fma(v.x, we.x, fma(v.y, we.y, acc[i].x));   // conj(v) * w
         acc[i].y = fma(v.x, we.y, fma(-v.y, we.x, acc[i].y));
       }
@@ -59,9 +60,10 @@ __global__ void k_mdot(long long n, int items, int nv, const double2* __restrict
   block_store(acc, nv, part, item, nblk);
 }
 
-__global__ void k_mupdate(long long n, int items, int nv, const double2* __restrict__ V,
-                          const double2* __restrict__ h, double2* __restrict__ w, double2* part,
+__global__ void k_mupdate(long long n, int items, int nv, const double2* V,
+                          const double2* h, double2* __restrict__ w, double2* part,
                           int nblk, int dot, double* nrm_part) {
+  pdl_enter();
   const int item = blockIdx.y;
   double2 hh[MAXV];
   for (int i = 0; i < MAXV; ++i) hh[i] = i < nv ? h[(long long)item * nv + i] : make_double2(0, 0);
@@ -75,7 +77,7 @@ __global__ void k_mupdate(long long n, int items, int nv, const double2* __restr
 #pragma unroll
     for (int i = 0; i < MAXV; ++i) {
       if (i < nv) {
-        vv[i] = __ldg(V + ((long long)i * items + item) * n + e);
+        vv[i] = *(V + ((long long)i * items + item) * n + e);
         we.x -= vv[i].x * hh[i].x - vv[i].y * hh[i].y;
         we.y -= vv[i].x * hh[i].y + vv[i].y * hh[i].x;
       }
@@ -106,12 +108,13 @@ __global__ void k_mupdate(long long n, int items, int nv, const double2* __restr
   }
 }
 
-__global__ void k_norm_part(long long n, const double2* __restrict__ w, double* part, int nblk) {
+__global__ void k_norm_part(long long n, const double2* w, double* part, int nblk) {
+  pdl_enter();
   const int item = blockIdx.y;
   const double2* wv = w + (long long)item * n;
   double nacc = 0.0;
   for (long long e = (long long)blockIdx.x * KB + threadIdx.x; e < n; e += (long long)nblk * KB) {
-    const double2 we = __ldg(wv + e);
+    const double2 we = *(wv + e);
     nacc = fma(we.x, we.x, fma(we.y, we.y, nacc));
   }
   __shared__ double shn[KB / 32];
@@ -126,8 +129,9 @@ __global__ void k_norm_part(long long n, const double2* __restrict__ w, double* 
 }
 
 // one warp per output: out[o] (+)= sum_blk part[o*nblk + blk]
-__global__ void k_reduce_parts(int nout, int nblk, const double2* __restrict__ part, double2* out,
+__global__ void k_reduce_parts(int nout, int nblk, const double2* part, double2* out,
                                int accumulate) {
+  pdl_enter();
   const int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (o >= nout) return;
@@ -142,7 +146,8 @@ __global__ void k_reduce_parts(int nout, int nblk, const double2* __restrict__ p
     out[o] = s;
   }
 }
-__global__ void k_reduce_norm(int items, int nblk, const double* __restrict__ part, double* out) {
+__global__ void k_reduce_norm(int items, int nblk, const double* part, double* out) {
+  pdl_enter();
   const int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (o >= items) return;
@@ -152,8 +157,9 @@ __global__ void k_reduce_norm(int items, int nblk, const double* __restrict__ pa
   if (lane == 0) out[o] = sqrt(s);
 }
 
-__global__ void k_scale_inv(long long n, const double2* __restrict__ w, const double* __restrict__ nrm,
+__global__ void k_scale_inv(long long n, const double2* w, const double* nrm,
                             double2* __restrict__ out) {
+  pdl_enter();
   const int item = blockIdx.y;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n) return;
@@ -162,19 +168,22 @@ __global__ void k_scale_inv(long long n, const double2* __restrict__ w, const do
   out[(long long)item * n + e] = make_double2(v.x * s, v.y * s);
 }
 
-__global__ void k_c128_c64(long long n, const double2* __restrict__ in, float2* __restrict__ out) {
+__global__ void k_c128_c64(long long n, const double2* in, float2* __restrict__ out) {
+  pdl_enter();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < n) { const double2 v = in[e]; out[e] = make_float2((float)v.x, (float)v.y); }
 }
-__global__ void k_c64_c128(long long n, const float2* __restrict__ in, double2* __restrict__ out) {
+__global__ void k_c64_c128(long long n, const float2* in, double2* __restrict__ out) {
+  pdl_enter();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < n) { const float2 v = in[e]; out[e] = make_double2(v.x, v.y); }
 }
 
 template <typename CZ>
-__global__ void k_xupdate(long long n, int items, int m, const CZ* __restrict__ Z,
-                          const double2* __restrict__ y, const int* __restrict__ kused,
+__global__ void k_xupdate(long long n, int items, int m, const CZ* Z,
+                          const double2* y, const int* kused,
                           double2* __restrict__ x) {
+  pdl_enter();
   const int item = blockIdx.y;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n) return;
@@ -201,32 +210,32 @@ int krylov_nblk(long long n) {
 
 void launch_mdot(long long n, int items, int nv, const double2* V, const double2* w, double2* part,
                  int nblk, cudaStream_t s) {
-  k_mdot<<<dim3(nblk, items), KB, 0, s>>>(n, items, nv, V, w, part, nblk);
+  launch_pdl(dim3(nblk, items), KB, 0, s, k_mdot, n, items, nv, V, w, part, nblk);
 }
 void launch_mupdate(long long n, int items, int nv, const double2* V, const double2* h, double2* w,
                     double2* part, int nblk, int dot, double* nrm_part, cudaStream_t s) {
-  k_mupdate<<<dim3(nblk, items), KB, 0, s>>>(n, items, nv, V, h, w, part, nblk, dot, nrm_part);
+  launch_pdl(dim3(nblk, items), KB, 0, s, k_mupdate, n, items, nv, V, h, w, part, nblk, dot, nrm_part);
 }
 void launch_reduce_parts(int items, int nv, int nblk, const double2* part, double2* out,
                          int accumulate, cudaStream_t s) {
   const int nout = items * nv;
-  k_reduce_parts<<<nb((long long)nout * 32, 128), 128, 0, s>>>(nout, nblk, part, out, accumulate);
+  launch_pdl(nb((long long)nout * 32, 128), 128, 0, s, k_reduce_parts, nout, nblk, part, out, accumulate);
 }
 void launch_norm_part(long long n, int items, const double2* w, double* part, int nblk, cudaStream_t s) {
-  k_norm_part<<<dim3(nblk, items), KB, 0, s>>>(n, w, part, nblk);
+  launch_pdl(dim3(nblk, items), KB, 0, s, k_norm_part, n, w, part, nblk);
 }
 void launch_reduce_norm(int items, int nblk, const double* part, double* out, cudaStream_t s) {
-  k_reduce_norm<<<nb((long long)items * 32, 128), 128, 0, s>>>(items, nblk, part, out);
+  launch_pdl(nb((long long)items * 32, 128), 128, 0, s, k_reduce_norm, items, nblk, part, out);
 }
 void launch_scale_inv(long long n, int items, const double2* w, const double* nrm, double2* out,
                       cudaStream_t s) {
-  k_scale_inv<<<dim3(nb(n, 256), items), 256, 0, s>>>(n, w, nrm, out);
+  launch_pdl(dim3(nb(n, 256), items), 256, 0, s, k_scale_inv, n, w, nrm, out);
 }
 void launch_cast_c128_c64(long long n, const double2* in, float2* out, cudaStream_t s) {
-  k_c128_c64<<<nb(n, 256), 256, 0, s>>>(n, in, out);
+  launch_pdl(nb(n, 256), 256, 0, s, k_c128_c64, n, in, out);
 }
 void launch_cast_c64_c128(long long n, const float2* in, double2* out, cudaStream_t s) {
-  k_c64_c128<<<nb(n, 256), 256, 0, s>>>(n, in, out);
+  launch_pdl(nb(n, 256), 256, 0, s, k_c64_c128, n, in, out);
 }
 void launch_copy(long long nbytes, const void* in, void* out, cudaStream_t s) {
   cudaMemcpyAsync(out, in, nbytes, cudaMemcpyDeviceToDevice, s);
@@ -234,7 +243,7 @@ void launch_copy(long long nbytes, const void* in, void* out, cudaStream_t s) {
 template <typename CZ>
 void launch_xupdate(long long n, int items, int m, const CZ* Z, const double2* y, const int* kused,
                     double2* x, cudaStream_t s) {
-  k_xupdate<CZ><<<dim3(nb(n, 256), items), 256, 0, s>>>(n, items, m, Z, y, kused, x);
+  launch_pdl(dim3(nb(n, 256), items), 256, 0, s, k_xupdate<CZ>, n, items, m, Z, y, kused, x);
 }
 template void launch_xupdate<float2>(long long, int, int, const float2*, const double2*, const int*,
                                      double2*, cudaStream_t);

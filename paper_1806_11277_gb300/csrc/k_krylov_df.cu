@@ -5,6 +5,10 @@
 // step is CGS2 (k_mdot_df, k_mupdate_df, k_update_scale_cast_df) or delayed
 // CGS2 (k_mdot2_df, k_dupdate_df).
 //
+// Launched plainly (a kernel starts when its inputs are complete), so that the passes over the basis may read it as
+// data that does not change (dfc_ld): with the plain loads of launch_pdl kernels the update pass took 52.9 us instead
+// of 37.5 (two media of 512^2).  The kernels of an Arnoldi step let their successors become resident early.
+//
 // Layouts: Krylov basis V and solution x as complex df64 (float4 per value),
 // preconditioned directions Z as complex64 (the multigrid cycle's output
 // precision), fine coefficients as 4 df64 reals per cell, coarsest inverse as
@@ -348,6 +352,7 @@ template <int NS>
 __global__ void __launch_bounds__(KB, 2) k_mdot2_df(long long n, int items, const float4* __restrict__ V,
                                                  const float4* __restrict__ w, float4* part, int nblk,
                                                  const int* __restrict__ il, int* cnt, float4* coef, double2* outd) {
+  pdl_trigger();
   constexpr int NO = NS + 1;   // NS dots and one norm per half
   static_assert(NO <= MAXV, "sums per half");
   const int item = il ? il[blockIdx.y] : blockIdx.y;
@@ -462,6 +467,7 @@ __global__ void __launch_bounds__(KB, 3) k_dupdate_df(long long n, int items, co
                                                    float4* vn, const float4* __restrict__ w,
                                                    const float4* __restrict__ coef, float2* __restrict__ out32,
                                                    const int* __restrict__ il) {
+  pdl_trigger();
   const int item = il ? il[blockIdx.y] : blockIdx.y;
   constexpr int NC = 2 * NJ + 3;
   static_assert(NC <= KDS, "coefficients per item");
@@ -705,6 +711,7 @@ __global__ void k_fine_apply_df2t(Grid g, int nrhs, const Coef4df* __restrict__ 
                                   const float2* __restrict__ vmt, FinePdf P, const V* __restrict__ x,
                                   const float4* __restrict__ b, float4* __restrict__ y, int mode,
                                   const int* __restrict__ il) {
+  pdl_trigger();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int item = il ? il[blockIdx.y] : blockIdx.y;
@@ -752,6 +759,7 @@ template <typename V, int D>
 __global__ void k_fine_apply_df(Grid g, int nrhs, const Coef4df* __restrict__ cf, FinePdf P,
                                 const V* __restrict__ x, const float4* __restrict__ b,
                                 float4* __restrict__ y, int mode, const int* __restrict__ il) {
+  pdl_trigger();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int item = il ? il[blockIdx.y] : blockIdx.y;
@@ -789,8 +797,8 @@ __device__ __forceinline__ void dacc2_fmaf(dacc2& a, float2 xh, float2 xl, float
   a.c = __fadd2_rn(a.c, __fadd2_rn(sg, pe));
 }
 __global__ void __launch_bounds__(256) k_dense_apply_df(int N, int nrhs, const float4* __restrict__ inv,
-                                                        const float2* __restrict__ r, float2* __restrict__ x,
-                                                        const int* __restrict__ il) {
+                                                        const float2* r, float2* __restrict__ x, const int* il) {
+  pdl_enter();
   constexpr int R = 2, U = 4;
   const int row0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * R;
   const int lane = threadIdx.x & 31;
@@ -813,7 +821,7 @@ __global__ void __launch_bounds__(256) k_dense_apply_df(int N, int nrhs, const f
       const bool in = j < N;
 #pragma unroll
       for (int k = 0; k < R; ++k) a[k][u] = in ? __ldg(m[k] + j) : z4;
-      b[u] = in ? __ldg(rv + j) : make_float2(0.f, 0.f);
+      b[u] = in ? rv[j] : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -979,7 +987,7 @@ void launch_dense_apply_df(int N, int items, int nrhs, const float4* inv, const 
                            cudaStream_t s) {
   const int bs = spread_bs((long long)(N + 1) / 2 * 32, items, 256);   // a warp per two rows
   const int rpb = bs / 32 * 2;
-  k_dense_apply_df<<<dim3((N + rpb - 1) / rpb, sel_items(items)), bs, 0, s>>>(N, nrhs, inv, r, x, g_sel.list);
+  launch_pdl(dim3((N + rpb - 1) / rpb, sel_items(items)), bs, 0, s, k_dense_apply_df, N, nrhs, inv, r, x, g_sel.list);
 }
 
 }  // namespace ehs

@@ -27,17 +27,18 @@ __device__ __forceinline__ void st_one_row(const Grid& g, const TT* ts, long lon
   Cx r = czero<Cx>();
   if (slot_valid(A, D, i)) {
     r = st_row_ct<T, TT, D, LV, SYM, A>(g, ts, c, i, xv);
-    if (mode) r = csub(__ldg(bv + (long long)A * N + c), r);
+    if (mode) r = csub(*(bv + (long long)A * N + c), r);
   }
   yv[(long long)A * N + c] = r;
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
 __global__ void __launch_bounds__(256) k_st_rows(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
-                                                 const typename CT<T>::type* __restrict__ x,
-                                                 const typename CT<T>::type* __restrict__ b,
+                                                 const typename CT<T>::type* x,
+                                                 const typename CT<T>::type* b,
                                                  typename CT<T>::type* __restrict__ y, int mode, int colour,
-                                                 const int* __restrict__ il) {
+                                                 const int* il) {
+  pdl_enter();
   constexpr StencilLayout L = level_layout(D, LV);
   const unsigned blk = blockIdx.x / (unsigned)nit, it = blockIdx.x - blk * (unsigned)nit;
   const long long c = (long long)blk * blockDim.x + threadIdx.x;
@@ -93,7 +94,7 @@ template <> struct Pair2<__nv_bfloat162> {
 template <typename T, typename TT, int D, int LV, bool SYM, int Q, int QE>
 __device__ __forceinline__ void row_acc2(typename CT<T>::type& y0, typename CT<T>::type& y1, const Grid& g,
                                          const TT* __restrict__ tab, long long c, const int i[3],
-                                         const typename CT<T>::type* __restrict__ x) {
+                                         const typename CT<T>::type* x) {
   if constexpr (Q < QE) {
     typedef typename CT<T>::type Cx;
     constexpr StencilLayout L = level_layout(D, LV);
@@ -135,8 +136,8 @@ __device__ __forceinline__ void row_acc2(typename CT<T>::type& y0, typename CT<T
           } else {
             Pair2<TT>::ld(tab + (long long)(base + ti) * N + c, t0, t1);
           }
-          if (in0) x0 = __ldg(xb + cj);
-          if (in1) x1 = __ldg(xb + cj + 1);
+          if (in0) x0 = *(xb + cj);
+          if (in1) x1 = *(xb + cj + 1);
           y0 = cfma(t0, x0, y0);
           y1 = cfma(t1, x1, y1);
         }
@@ -160,17 +161,18 @@ __device__ __forceinline__ void st_two_rows(const Grid& g, const TT* ts, long lo
   const int par = (i[0] + i[1] + i[2]) & 1;
   const bool w0 = !(A == D && colour >= 0 && par != colour), w1 = !(A == D && colour >= 0 && par == colour);
   if (mode) {
-    if (v0) y0 = csub(__ldg(bv + (long long)A * N + c), y0);
-    if (v1) y1 = csub(__ldg(bv + (long long)A * N + c + 1), y1);
+    if (v0) y0 = csub(*(bv + (long long)A * N + c), y0);
+    if (v1) y1 = csub(*(bv + (long long)A * N + c + 1), y1);
   }
   if (w0) yv[(long long)A * N + c] = v0 ? y0 : czero<Cx>();
   if (w1) yv[(long long)A * N + c + 1] = v1 ? y1 : czero<Cx>();
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
-__global__ void k_st_rows2(Grid g, int nit, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* __restrict__ x,
-                           const typename CT<T>::type* __restrict__ b, typename CT<T>::type* __restrict__ y,
-                           int mode, int colour, const int* __restrict__ il) {
+__global__ void k_st_rows2(Grid g, int nit, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* x,
+                           const typename CT<T>::type* b, typename CT<T>::type* __restrict__ y,
+                           int mode, int colour, const int* il) {
+  pdl_enter();
   constexpr StencilLayout L = level_layout(D, LV);
   const unsigned blk = blockIdx.x / (unsigned)nit, it = blockIdx.x - blk * (unsigned)nit;
   const long long t = (long long)blk * blockDim.x + threadIdx.x;
@@ -207,20 +209,20 @@ static void st_apply_t(const Grid& g, int items, int nrhs, int v, const TT* tab,
   if (kRowsCpt[var] == 1) {
     const dim3 gr((unsigned)((g.ncell + bs - 1) / bs) * nit, 1, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) k_st_rows<T, TT, 2, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows<T, TT, 2, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     } else if constexpr (!SYM) {
-      if (v == 1) k_st_rows<T, TT, 3, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows<T, TT, 3, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     }
   } else {
     const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs) * nit, 1, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) k_st_rows2<T, TT, 2, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows2<T, TT, 2, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     } else if constexpr (!SYM) {
-      if (v == 1) k_st_rows2<T, TT, 3, 1, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else k_st_rows2<T, TT, 3, 2, SYM><<<gr, bs, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     }
   }
 }

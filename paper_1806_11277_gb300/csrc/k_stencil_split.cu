@@ -69,7 +69,7 @@ __constant__ LineTab kLines[2] = {make_lines(1), make_lines(2)};   // level 1, l
 template <typename T, typename TT, int NS>
 __device__ __forceinline__ typename CT<T>::type row_lines(const Grid& g, const LineTab& LT, const TT* __restrict__ ts,
                                                           long long c, const int i[3],
-                                                          const typename CT<T>::type* __restrict__ x, int a, int part) {
+                                                          const typename CT<T>::type* x, int a, int part) {
   typedef typename CT<T>::type Cx;
   const long long N = g.ncell, sy = g.n[0], sz = (long long)g.n[0] * g.n[1];
   Cx y = czero<Cx>();
@@ -86,7 +86,7 @@ __device__ __forceinline__ typename CT<T>::type row_lines(const Grid& g, const L
       tv[k] = xv[k] = czero<Cx>();
       if (k < R.len && rin && jx + k >= 0 && jx + k < g.n[0]) {
         tv[k] = ldtab<T>(tp + k * N);
-        xv[k] = __ldg(xp + k);
+        xv[k] = *(xp + k);
       }
     }
 #pragma unroll
@@ -120,10 +120,11 @@ __device__ __forceinline__ typename CT<T>::type row_share(const Grid& g, const T
 
 template <typename T, typename TT, int D, int LV, bool SYM, int NS>
 __global__ void __launch_bounds__(32 * NS) k_st_rows_split(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
-                                                           const typename CT<T>::type* __restrict__ x,
-                                                           const typename CT<T>::type* __restrict__ b,
+                                                           const typename CT<T>::type* x,
+                                                           const typename CT<T>::type* b,
                                                            typename CT<T>::type* __restrict__ y, int mode, int colour,
-                                                           const int* __restrict__ il) {
+                                                           const int* il) {
+  pdl_enter();
   typedef typename CT<T>::type Cx;
   constexpr StencilLayout L = level_layout(D, LV);
   constexpr int nslot = SYM ? half_base(L, L.npair) : L.nslot;
@@ -147,17 +148,20 @@ __global__ void __launch_bounds__(32 * NS) k_st_rows_split(Grid g, int nit, int 
   Cx r = sp[0][lane];
 #pragma unroll
   for (int q = 1; q < NS; ++q) r = cadd(r, sp[q][lane]);
-  if (mode && row) r = csub(__ldg(b + vo + (long long)a * N + c), r);
+  if (mode && row) r = csub(*(b + vo + (long long)a * N + c), r);
   y[vo + (long long)a * N + c] = r;
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM, int NS>
 __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int nit, int nrhs,
-                                                                     const TT* __restrict__ tab, T wu, T wp, int colour,
-                                                                     const typename CT<T>::type* __restrict__ b,
-                                                                     const typename CT<T>::type* __restrict__ xi,
+                                                                     const TT* __restrict__ tab,
+                                                                     const typename CT<T>::type* __restrict__ vtab,
+                                                                     T wu, T wp, int colour,
+                                                                     const typename CT<T>::type* b,
+                                                                     const typename CT<T>::type* xi,
                                                                      typename CT<T>::type* __restrict__ xo,
-                                                                     const int* __restrict__ il) {
+                                                                     const int* il) {
+  pdl_trigger();
   typedef typename CT<T>::type Cx;
   constexpr StencilLayout L = level_layout(D, LV);
   constexpr int NB = 2 * D + 1;
@@ -177,24 +181,35 @@ __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int
     cell_coords(g, c, i);
     if (((i[0] + i[1] + i[2]) & 1) != colour) { ++c; ++i[0]; }
   }
-  // the first warp: block coefficients, right-hand sides and the old iterate, in flight while the rows are summed
-  Cx r[NB], dg[2 * D], gr[2 * D], gc[2 * D], sch = czero<Cx>(), xv[NB];
+  // the first warp: block coefficients (setup-time data, before the wait), then right-hand sides and the old
+  // iterate, in flight while the rows are summed
+  const Cx* vt = vtab + (long long)(item / nrhs) * (D + 1) * N;
+  Cx r[NB], dinv[2 * D], gr[2 * D], gc[2 * D], sinv = czero<Cx>(), xv[NB], po = czero<Cx>();
   bool ok[2 * D];
+  const long long co = (c & 1) ? c - 1 : c + 1;
+  if (wid == 0 && live) {
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      ok[k] = i[k] >= 1;
+      ok[D + k] = i[k] + 1 < g.n[k];
+    }
+    vupd_coefs<T, TT, D, LV, SYM, 0>(ts, vt, N, c, stride_of(g, 0), ok[0], ok[D], dinv, gr, gc);
+    vupd_coefs<T, TT, D, LV, SYM, 1>(ts, vt, N, c, stride_of(g, 1), ok[1], ok[D + 1], dinv, gr, gc);
+    if constexpr (D == 3)
+      vupd_coefs<T, TT, D, LV, SYM, 2>(ts, vt, N, c, stride_of(g, 2), ok[2], ok[D + 2], dinv, gr, gc);
+    sinv = __ldg(vt + (long long)D * N + c);
+  }
+  pdl_wait();
   if (wid == 0 && live) {
 #pragma unroll
     for (int k = 0; k < D; ++k) {
       const long long lo = (long long)k * N + c, hi = lo + stride_of(g, k);
-      ok[k] = i[k] >= 1;
-      ok[D + k] = i[k] + 1 < g.n[k];
-      if (ok[k]) { r[k] = __ldg(b + vo + lo); xv[k] = __ldg(x + lo); }
-      if (ok[D + k]) { r[D + k] = __ldg(b + vo + hi); xv[D + k] = __ldg(x + hi); }
+      if (ok[k]) { r[k] = b[vo + lo]; xv[k] = x[lo]; }
+      if (ok[D + k]) { r[D + k] = b[vo + hi]; xv[D + k] = x[hi]; }
     }
-    r[2 * D] = __ldg(b + vo + (long long)D * N + c);
-    xv[2 * D] = __ldg(x + (long long)D * N + c);
-    vupd_coefs<T, TT, D, LV, SYM, 0>(ts, N, c, stride_of(g, 0), ok[0], ok[D], dg, gr, gc);
-    vupd_coefs<T, TT, D, LV, SYM, 1>(ts, N, c, stride_of(g, 1), ok[1], ok[D + 1], dg, gr, gc);
-    if constexpr (D == 3) vupd_coefs<T, TT, D, LV, SYM, 2>(ts, N, c, stride_of(g, 2), ok[2], ok[D + 2], dg, gr, gc);
-    sch = tab_coef<T, TT, D, LV, SYM, D, D, 0, 0, 0>(ts, N, c, 0);
+    r[2 * D] = b[vo + (long long)D * N + c];
+    xv[2 * D] = x[(long long)D * N + c];
+    po = x[(long long)D * N + co];
   }
   {  // this warp's share of one row of the cell's block
     const int k = row % D;
@@ -212,9 +227,8 @@ __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int
   __syncthreads();
   if (wid || !live) return;
   Cx* xout = xo + vo;
-  const long long co = (c & 1) ? c - 1 : c + 1;
-  xout[(long long)D * N + co] = __ldg(x + (long long)D * N + co);
-  Cx rp = r[2 * D], dinv[2 * D];
+  xout[(long long)D * N + co] = po;
+  Cx rp = r[2 * D];
 #pragma unroll
   for (int a = 0; a < NB; ++a) {
     Cx s = sp[a][0][lane];
@@ -224,14 +238,9 @@ __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int
     else if (ok[a]) r[a] = csub(r[a], s);
   }
 #pragma unroll
-  for (int a = 0; a < 2 * D; ++a) {
-    if (!ok[a]) continue;
-    dinv[a] = cinv(dg[a]);
-    const Cx gd = cmul(gc[a], dinv[a]);
-    sch = csub(sch, cmul(gd, gr[a]));
-    rp = csub(rp, cmul(gd, r[a]));
-  }
-  const Cx dp = cmul(rp, cinv(sch));
+  for (int a = 0; a < 2 * D; ++a)
+    if (ok[a]) rp = csub(rp, cmul(cmul(gc[a], dinv[a]), r[a]));
+  const Cx dp = cmul(rp, sinv);
   xout[(long long)D * N + c] = cfma(mk<T>(wp, 0), dp, xv[2 * D]);
 #pragma unroll
   for (int a = 0; a < 2 * D; ++a) {
@@ -249,10 +258,11 @@ __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int
 template <typename T, typename TT, int LV>
 __global__ void __launch_bounds__(256) k_st_gather3(Grid g, int nrhs, int nsub, int nloc, const int* __restrict__ map,
                                                     const TT* __restrict__ tab,
-                                                    const typename CT<T>::type* __restrict__ x,
-                                                    const typename CT<T>::type* __restrict__ b,
+                                                    const typename CT<T>::type* x,
+                                                    const typename CT<T>::type* b,
                                                     typename CT<T>::type* __restrict__ out,
-                                                    const int* __restrict__ il) {
+                                                    const int* il) {
+  pdl_enter();
   typedef typename CT<T>::type Cx;
   constexpr int nslot = level_layout(3, LV).nslot;
   constexpr int NS = 8;
@@ -275,7 +285,7 @@ __global__ void __launch_bounds__(256) k_st_gather3(Grid g, int nrhs, int nsub, 
   if (part || e >= nloc) return;
 #pragma unroll
   for (int q = 1; q < NS; ++q) v = cadd(v, sp[q][lane]);
-  if (gs >= 0) v = csub(__ldg(b + vo + gs), v);
+  if (gs >= 0) v = csub(*(b + vo + gs), v);
   out[(long long)bl * nloc + e] = v;
 }
 
@@ -304,7 +314,7 @@ void rows_split_t(const Grid& g, int items, int nrhs, const TT* tab, const typen
   constexpr int NS = Ns<D>::rows;
   const int nit = (int)sel_items(items);
   const dim3 gr((unsigned)((g.ncell + 31) / 32) * nit, 1, D + 1);
-  k_st_rows_split<T, TT, D, LV, SYM, NS><<<gr, 32 * NS, 0, s>>>(g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+  launch_pdl(gr, 32 * NS, 0, s, k_st_rows_split<T, TT, D, LV, SYM, NS>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
 }
 template <typename T, typename TT, bool SYM>
 void rows_split_d(int v, const TT* tab, const Grid& g, int items, int nrhs, const typename CT<T>::type* x,
@@ -322,24 +332,24 @@ void gather3_d(int v, const TT* tab, const Grid& g, int items_l, int nrhs, int n
                const typename CT<T>::type* x, const typename CT<T>::type* b, typename CT<T>::type* out, cudaStream_t s) {
   if constexpr (!SYM) {
     const dim3 gr((unsigned)((nloc + 31) / 32), sel_items(items_l));
-    if (v == 1) k_st_gather3<T, TT, 1><<<gr, 256, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
-    else k_st_gather3<T, TT, 2><<<gr, 256, 0, s>>>(g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
+    if (v == 1) launch_pdl(gr, 256, 0, s, k_st_gather3<T, TT, 1>, g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
+    else launch_pdl(gr, 256, 0, s, k_st_gather3<T, TT, 2>, g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
   }
 }
 template <typename TT, int LV, bool SYM>
-void colour_t(const Grid& g, int items, int nrhs, const TT* tab, float wu, float wp, int colour, const float2* b,
+void colour_t(const Grid& g, int items, int nrhs, const TT* tab, const float2* vt, float wu, float wp, int colour, const float2* b,
               const float2* xi, float2* xo, cudaStream_t s) {
   constexpr int NS = Ns<2>::colour;
   const int nit = (int)sel_items(items);
   const dim3 gr((unsigned)((g.ncell / 2 + 31) / 32) * nit);
-  k_st_colour<float, TT, 2, LV, SYM, NS><<<gr, 32 * 5 * NS, 0, s>>>(g, nit, nrhs, tab, wu, wp, colour, b, xi, xo,
+  launch_pdl(gr, 32 * 5 * NS, 0, s, k_st_colour<float, TT, 2, LV, SYM, NS>, g, nit, nrhs, tab, vt, wu, wp, colour, b, xi, xo,
                                                                     g_sel.list);
 }
 template <typename T, typename TT, bool SYM>
-void colour_d(int v, const TT* tab, const Grid& g, int items, int nrhs, float wu, float wp, int colour, const float2* b,
-              const float2* xi, float2* xo, cudaStream_t s) {
-  if (v == 1) colour_t<TT, 1, SYM>(g, items, nrhs, tab, wu, wp, colour, b, xi, xo, s);
-  else colour_t<TT, 2, SYM>(g, items, nrhs, tab, wu, wp, colour, b, xi, xo, s);
+void colour_d(int v, const TT* tab, const Grid& g, int items, int nrhs, const float2* vt, float wu, float wp, int colour,
+              const float2* b, const float2* xi, float2* xo, cudaStream_t s) {
+  if (v == 1) colour_t<TT, 1, SYM>(g, items, nrhs, tab, vt, wu, wp, colour, b, xi, xo, s);
+  else colour_t<TT, 2, SYM>(g, items, nrhs, tab, vt, wu, wp, colour, b, xi, xo, s);
 }
 
 }  // namespace
@@ -366,10 +376,10 @@ void launch_st_rows_split(const Grid& g, int items, int nrhs, int v, const void*
                           int mode, int colour, cudaStream_t s) {
   EHS_ST_FORMATS(rows_split_d, g, items, nrhs, x, b, y, mode, colour, s);
 }
-void launch_st_colour(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt, float wu, float wp, int colour,
-                      const float2* b, const float2* xi, float2* xo, cudaStream_t s) {
+void launch_st_colour(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt, const float2* vt, float wu,
+                      float wp, int colour, const float2* b, const float2* xi, float2* xo, cudaStream_t s) {
   typedef float T;
-  EHS_ST_FORMATS(colour_d, g, items, nrhs, wu, wp, colour, b, xi, xo, s);
+  EHS_ST_FORMATS(colour_d, g, items, nrhs, vt, wu, wp, colour, b, xi, xo, s);
 }
 
 template <typename T>

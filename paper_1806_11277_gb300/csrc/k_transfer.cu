@@ -45,8 +45,9 @@ template <typename T, typename C> __device__ __forceinline__ C rfma(T w, C v, C 
 
 // thread per coarse cell and component: fine offsets -1..2 around 2 I along every direction
 template <typename T, int D>
-__global__ void k_restrict(Grid gf, Grid gc, const typename CT<T>::type* __restrict__ rf,
-                           typename CT<T>::type* __restrict__ rc, const int* __restrict__ il) {
+__global__ void k_restrict(Grid gf, Grid gc, const typename CT<T>::type* rf,
+                           typename CT<T>::type* __restrict__ rc, const int* il) {
+  pdl_enter();
   typedef typename CT<T>::type C;
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= gc.ncell) return;
@@ -75,7 +76,7 @@ __global__ void k_restrict(Grid gf, Grid gc, const typename CT<T>::type* __restr
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
           C v = czero<C>();
-          if (yin && q[0][x] != 0) v = __ldg(row + x);
+          if (yin && q[0][x] != 0) v = *(row + x);
           rs = rfma(quarters<T>(q[0][x]), v, rs);
         }
         pl = rfma(quarters<T>(q[1][y]), rs, pl);
@@ -88,8 +89,9 @@ __global__ void k_restrict(Grid gf, Grid gc, const typename CT<T>::type* __restr
 
 // thread per fine cell and component: at most two coarse indices per direction (pw_pair)
 template <typename T, int D>
-__global__ void k_prolong_add(Grid gf, Grid gc, const typename CT<T>::type* __restrict__ ec,
-                              typename CT<T>::type* __restrict__ xf, const int* __restrict__ il) {
+__global__ void k_prolong_add(Grid gf, Grid gc, const typename CT<T>::type* ec,
+                              typename CT<T>::type* __restrict__ xf, const int* il) {
+  pdl_enter();
   typedef typename CT<T>::type C;
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= gf.ncell) return;
@@ -122,7 +124,7 @@ __global__ void k_prolong_add(Grid gf, Grid gc, const typename CT<T>::type* __re
 #pragma unroll
       for (int xx = 0; xx < 2; ++xx) {
         C v = czero<C>();
-        if (yin && q[0][xx] != 0) v = __ldg(row + J[0][xx]);
+        if (yin && q[0][xx] != 0) v = *(row + J[0][xx]);
         rs = rfma(quarters<T>(q[0][xx]), v, rs);
       }
       pl = rfma(quarters<T>(q[1][y]), rs, pl);
@@ -139,8 +141,8 @@ void launch_restrict(const Grid& gf, const Grid& gc, int items, const typename C
                      typename CT<T>::type* rc, cudaStream_t s) {
   const int bs = spread_bs(gc.ncell * (gf.d + 1), items, 128);
   const dim3 gr((unsigned)((gc.ncell + bs - 1) / bs), sel_items(items), gf.d + 1);
-  if (gf.d == 2) k_restrict<T, 2><<<gr, bs, 0, s>>>(gf, gc, rf, rc, g_sel.list);
-  else k_restrict<T, 3><<<gr, bs, 0, s>>>(gf, gc, rf, rc, g_sel.list);
+  if (gf.d == 2) launch_pdl(gr, bs, 0, s, k_restrict<T, 2>, gf, gc, rf, rc, g_sel.list);
+  else launch_pdl(gr, bs, 0, s, k_restrict<T, 3>, gf, gc, rf, rc, g_sel.list);
 }
 
 template <typename T>
@@ -148,8 +150,8 @@ void launch_prolong_add(const Grid& gf, const Grid& gc, int items, const typenam
                         typename CT<T>::type* xf, cudaStream_t s) {
   const int bs = spread_bs(gf.ncell * (gf.d + 1), items, 256);
   const dim3 gr((unsigned)((gf.ncell + bs - 1) / bs), sel_items(items), gf.d + 1);
-  if (gf.d == 2) k_prolong_add<T, 2><<<gr, bs, 0, s>>>(gf, gc, ec, xf, g_sel.list);
-  else k_prolong_add<T, 3><<<gr, bs, 0, s>>>(gf, gc, ec, xf, g_sel.list);
+  if (gf.d == 2) launch_pdl(gr, bs, 0, s, k_prolong_add<T, 2>, gf, gc, ec, xf, g_sel.list);
+  else launch_pdl(gr, bs, 0, s, k_prolong_add<T, 3>, gf, gc, ec, xf, g_sel.list);
 }
 
 #define INST(T)                                                                                 \

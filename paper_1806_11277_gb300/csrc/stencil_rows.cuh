@@ -59,7 +59,7 @@ template <typename T, typename TT, int D, int LV, bool SYM, int Q, int QE, bool 
 __device__ __forceinline__ void row_acc(typename CT<T>::type& y, const Grid& g,
                                         const TT* __restrict__ tab,
                                         long long c, const int i[3],
-                                        const typename CT<T>::type* __restrict__ x) {
+                                        const typename CT<T>::type* x) {
   if constexpr (Q < QE) {
     constexpr StencilLayout L = level_layout(D, LV);
     constexpr int b = L.p[Q].b, base = L.p[Q].base;
@@ -95,7 +95,7 @@ __device__ __forceinline__ void row_acc(typename CT<T>::type& y, const Grid& g,
             } else {
               tv = ldtab<T>(tab + (long long)(base + ti) * N + c);
             }
-            if (in) xv = XCG ? __ldcg(xb + cj) : __ldg(xb + cj);
+            if (in) xv = XCG ? __ldcg(xb + cj) : *(xb + cj);
             y = cfma(tv, xv, y);
           }
         }
@@ -134,20 +134,22 @@ __device__ __forceinline__ typename CT<T>::type tab_coef(const TT* ts, long long
   }
 }
 
-// the block coefficients of component K of the economic cell update: diagonals of the low
-// and high face, their couplings to the cell's pressure, and back
+// The block coefficients of component K of the economic cell update: couplings of the low and high face to the
+// cell's pressure (gr) and back (gc), and the inverses of the two diagonals (dinv), from the setup-time table vt
+// ([D + 1][ncell] of one medium: inverse diagonals of the low face rows, then the blocks' inverse Schur
+// complements; launch_vupd_tab).
 template <typename T, typename TT, int D, int LV, bool SYM, int K>
-__device__ __forceinline__ void vupd_coefs(const TT* ts, long long N, long long c, long long sk, bool lo_ok,
-                                           bool hi_ok, typename CT<T>::type* dg, typename CT<T>::type* gr,
-                                           typename CT<T>::type* gc) {
+__device__ __forceinline__ void vupd_coefs(const TT* ts, const typename CT<T>::type* vt, long long N, long long c,
+                                           long long sk, bool lo_ok, bool hi_ok, typename CT<T>::type* dinv,
+                                           typename CT<T>::type* gr, typename CT<T>::type* gc) {
   constexpr int E0 = K == 0, E1 = K == 1, E2 = K == 2;
   if (lo_ok) {
-    dg[K] = tab_coef<T, TT, D, LV, SYM, K, K, 0, 0, 0>(ts, N, c, 0);
+    dinv[K] = __ldg(vt + (long long)K * N + c);
     gr[K] = tab_coef<T, TT, D, LV, SYM, K, D, 0, 0, 0>(ts, N, c, 0);
     gc[K] = tab_coef<T, TT, D, LV, SYM, D, K, 0, 0, 0>(ts, N, c, 0);
   }
   if (hi_ok) {
-    dg[D + K] = tab_coef<T, TT, D, LV, SYM, K, K, 0, 0, 0>(ts, N, c + sk, 0);
+    dinv[D + K] = __ldg(vt + (long long)K * N + c + sk);
     gr[D + K] = tab_coef<T, TT, D, LV, SYM, K, D, -E0, -E1, -E2>(ts, N, c + sk, -sk);
     gc[D + K] = tab_coef<T, TT, D, LV, SYM, D, K, E0, E1, E2>(ts, N, c, sk);
   }
