@@ -64,35 +64,40 @@ __host__ __device__ constexpr bool lines_ok(const LineTab& T) {
 static_assert(lines_ok(make_lines(1)) && lines_ok(make_lines(2)), "line tables");
 __constant__ LineTab kLines[2] = {make_lines(1), make_lines(2)};   // level 1, level 2 on
 
-// lines part, part + NS, ... of row a at cell c: a loop over the lines (read from constant memory, the same for the
-// whole warp), each line's loads in flight together
-template <typename T, typename TT, int NS>
-__device__ __forceinline__ typename CT<T>::type row_lines(const Grid& g, const LineTab& LT, const TT* __restrict__ ts,
-                                                          long long c, const int i[3],
-                                                          const typename CT<T>::type* x, int a, int part) {
+// lines part, part + NS, ... of row a at cell c for NI vectors: a loop over the lines (read from constant memory, the
+// same for the whole warp), each line's loads in flight together
+template <typename T, typename TT, int NS, int NI>
+__device__ __forceinline__ void row_lines(const Grid& g, const LineTab& LT, const TT* __restrict__ ts, long long c,
+                                          const int i[3], const typename CT<T>::type* const (&x)[NI], int a, int part,
+                                          typename CT<T>::type (&y)[NI]) {
   typedef typename CT<T>::type Cx;
   const long long N = g.ncell, sy = g.n[0], sz = (long long)g.n[0] * g.n[1];
-  Cx y = czero<Cx>();
+#pragma unroll
+  for (int q = 0; q < NI; ++q) y[q] = czero<Cx>();
 #pragma unroll 2
   for (int l = LT.first[a] + part; l < LT.first[a + 1]; l += NS) {
     const Line& R = LT.l[l];
     const int jy = i[1] + R.oy, jz = i[2] + R.oz, jx = i[0] + R.ox0;
     const bool rin = jy >= 0 && jy < g.n[1] && jz >= 0 && jz < g.n[2];
-    const Cx* xp = x + R.b * N + (c + R.oz * sz + R.oy * sy + R.ox0);
+    const long long xo = R.b * N + (c + R.oz * sz + R.oy * sy + R.ox0);
     const TT* tp = ts + R.slot0 * N + c;
-    Cx tv[MAXLEN], xv[MAXLEN];
+    Cx tv[MAXLEN], xv[NI][MAXLEN];
 #pragma unroll
     for (int k = 0; k < MAXLEN; ++k) {
-      tv[k] = xv[k] = czero<Cx>();
+      tv[k] = czero<Cx>();
+#pragma unroll
+      for (int q = 0; q < NI; ++q) xv[q][k] = czero<Cx>();
       if (k < R.len && rin && jx + k >= 0 && jx + k < g.n[0]) {
         tv[k] = ldtab<T>(tp + k * N);
-        xv[k] = *(xp + k);
+#pragma unroll
+        for (int q = 0; q < NI; ++q) xv[q][k] = x[q][xo + k];
       }
     }
 #pragma unroll
-    for (int k = 0; k < MAXLEN; ++k) y = cfma(tv[k], xv[k], y);
+    for (int k = 0; k < MAXLEN; ++k)
+#pragma unroll
+      for (int q = 0; q < NI; ++q) y[q] = cfma(tv[k], xv[q][k], y[q]);
   }
-  return y;
 }
 
 // the share `part` of NS of row a at cell c, unrolled (2D)
@@ -109,13 +114,10 @@ __device__ __forceinline__ typename CT<T>::type row_part(const Grid& g, const TT
 template <typename T, typename TT, int D, int LV, bool SYM, int NS>
 __device__ __forceinline__ typename CT<T>::type row_share(const Grid& g, const TT* ts, long long c, const int i[3],
                                                           const typename CT<T>::type* x, int a, int part) {
-  if constexpr (D == 3) {
-    return row_lines<T, TT, NS>(g, kLines[LV - 1], ts, c, i, x, a, part);
-  } else {
-    if (a == 0) return row_part<T, TT, LV, SYM, NS, 0>(g, ts, c, i, x, part);
-    if (a == 1) return row_part<T, TT, LV, SYM, NS, 1>(g, ts, c, i, x, part);
-    return row_part<T, TT, LV, SYM, NS, 2>(g, ts, c, i, x, part);
-  }
+  static_assert(D == 2, "3D rows go by lines");
+  if (a == 0) return row_part<T, TT, LV, SYM, NS, 0>(g, ts, c, i, x, part);
+  if (a == 1) return row_part<T, TT, LV, SYM, NS, 1>(g, ts, c, i, x, part);
+  return row_part<T, TT, LV, SYM, NS, 2>(g, ts, c, i, x, part);
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM, int NS>
@@ -150,6 +152,73 @@ __global__ void __launch_bounds__(32 * NS) k_st_rows_split(Grid g, int nit, int 
   for (int q = 1; q < NS; ++q) r = cadd(r, sp[q][lane]);
   if (mode && row) r = csub(*(b + vo + (long long)a * N + c), r);
   y[vo + (long long)a * N + c] = r;
+}
+
+// The 3D form: NI items of the list per block, one read of the table for all of them where they are of one medium
+// (its coefficients are nine tenths of the bytes; 64^3, complex64 tables, two sources, mean of levels 1 and 2: 43 us with an
+// item a block, the table read once per item -> 30 us).
+template <typename T, typename TT, int LV, int NS, int NI>
+__global__ void __launch_bounds__(32 * NS) k_st_rows_split3(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
+                                                            const typename CT<T>::type* x,
+                                                            const typename CT<T>::type* b,
+                                                            typename CT<T>::type* __restrict__ y, int mode, int colour,
+                                                            const int* il) {
+  pdl_enter();
+  typedef typename CT<T>::type Cx;
+  constexpr int nslot = level_layout(3, LV).nslot;
+  __shared__ Cx sp[NI][NS][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, a = blockIdx.z;
+  const unsigned ng = (nit + NI - 1) / NI, blk = blockIdx.x / ng, it0 = (blockIdx.x - blk * ng) * NI;
+  const long long c = (long long)blk * 32 + lane, N = g.ncell;
+  int item[NI], live = 0;
+  bool same = true;
+#pragma unroll
+  for (int q = 0; q < NI; ++q) {
+    item[q] = item[0];
+    if ((int)it0 + q < nit) { item[q] = il ? il[it0 + q] : it0 + q; ++live; }
+    same = same && item[q] / nrhs == item[0] / nrhs;
+  }
+  int i[3] = {0, 0, 0};
+  bool run = c < N;
+  if (run) {
+    cell_coords(g, c, i);
+    run = !(a == 3 && colour >= 0 && ((i[0] + i[1] + i[2]) & 1) != colour);
+  }
+  const bool row = run && slot_valid(a, 3, i);
+  const Cx* xs[NI];
+#pragma unroll
+  for (int q = 0; q < NI; ++q) xs[q] = x + (long long)item[q] * 4 * N;
+  Cx v[NI];
+#pragma unroll
+  for (int q = 0; q < NI; ++q) v[q] = czero<Cx>();
+  if (row) {
+    if (same) {
+      row_lines<T, TT, NS, NI>(g, kLines[LV - 1], tab + (long long)(item[0] / nrhs) * nslot * N, c, i, xs, a, part, v);
+    } else {
+      for (int q = 0; q < live; ++q) {
+        const Cx* x1[1] = {x + (long long)item[q] * 4 * N};
+        Cx y1[1];
+        row_lines<T, TT, NS, 1>(g, kLines[LV - 1], tab + (long long)(item[q] / nrhs) * nslot * N, c, i, x1, a, part, y1);
+#pragma unroll
+        for (int p = 0; p < NI; ++p)
+          if (p == q) v[p] = y1[0];
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NI; ++q) sp[q][part][lane] = v[q];
+  __syncthreads();
+  if (part >= live || !run) return;      // warp q finishes item q
+  Cx r = sp[part][0][lane];
+#pragma unroll
+  for (int q = 1; q < NS; ++q) r = cadd(r, sp[part][q][lane]);
+  int it = item[0];
+#pragma unroll
+  for (int q = 1; q < NI; ++q)
+    if (part == q) it = item[q];
+  const long long o = ((long long)it * 4 + a) * N + c;
+  if (mode && row) r = csub(b[o], r);
+  y[o] = r;
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM, int NS>
@@ -278,7 +347,10 @@ __global__ void __launch_bounds__(256) k_st_gather3(Grid g, int nrhs, int nsub, 
     const int a = gs / (int)N, c = gs - a * (int)N;
     int i[3];
     cell_coords(g, c, i);
-    v = row_lines<T, TT, NS>(g, kLines[LV - 1], tab + (long long)m * nslot * N, c, i, x + vo, a, part);
+    const Cx* xs[1] = {x + vo};
+    Cx y[1];
+    row_lines<T, TT, NS, 1>(g, kLines[LV - 1], tab + (long long)m * nslot * N, c, i, xs, a, part, y);
+    v = y[0];
   }
   sp[part][lane] = v;
   __syncthreads();
@@ -313,8 +385,18 @@ void rows_split_t(const Grid& g, int items, int nrhs, const TT* tab, const typen
                   const typename CT<T>::type* b, typename CT<T>::type* y, int mode, int colour, cudaStream_t s) {
   constexpr int NS = Ns<D>::rows;
   const int nit = (int)sel_items(items);
-  const dim3 gr((unsigned)((g.ncell + 31) / 32) * nit, 1, D + 1);
-  launch_pdl(gr, 32 * NS, 0, s, k_st_rows_split<T, TT, D, LV, SYM, NS>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+  const unsigned nb = (unsigned)((g.ncell + 31) / 32);
+  if constexpr (D == 3) {
+    if (nrhs > 1)
+      launch_pdl(dim3(nb * ((nit + 1) / 2), 1, 4), 32 * NS, 0, s, k_st_rows_split3<T, TT, LV, NS, 2>, g, nit, nrhs, tab, x,
+                 b, y, mode, colour, g_sel.list);
+    else
+      launch_pdl(dim3(nb * nit, 1, 4), 32 * NS, 0, s, k_st_rows_split3<T, TT, LV, NS, 1>, g, nit, nrhs, tab, x, b, y, mode,
+                 colour, g_sel.list);
+  } else {
+    launch_pdl(dim3(nb * nit, 1, 3), 32 * NS, 0, s, k_st_rows_split<T, TT, D, LV, SYM, NS>, g, nit, nrhs, tab, x, b, y,
+               mode, colour, g_sel.list);
+  }
 }
 template <typename T, typename TT, bool SYM>
 void rows_split_d(int v, const TT* tab, const Grid& g, int items, int nrhs, const typename CT<T>::type* x,
