@@ -1386,7 +1386,7 @@ ehs_status ehs_create(const ehs_problem* prob, const ehs_opts* opts, void* strea
     // Krylov workspace
     const int m = opts->restart, items = H.items;
     const long long n = c->n0;
-    c->nblk = krylov_nblk(n);
+    c->nblk = krylov_nblk(n, items);
     c->V = dalloc<double2>(c, (size_t)(m + 1) * items * n);
     c->Z = dalloc<double2>(c, (size_t)m * items * n);
     c->w = dalloc<double2>(c, (size_t)items * n);

@@ -910,8 +910,12 @@ void launch_mdot2_df(long long n, int items, int j, const float4* V, const float
 }
 void launch_dupdate_df(long long n, int items, int j, float4* V, const float4* w, const float4* coef,
                        float2* out32, cudaStream_t s) {
-  long long gb = (n + KB - 1) / KB;   // as launch_update_scale_cast_df: 3 CTAs per SM, one wave per item
-  if (gb > 3 * 152) gb = 3 * 152;
+  // 3 CTAs per SM: one wave for an item alone; in a batch a thread keeps at least four elements (16 sources of 256^2:
+  // 79 us a launch with a wave per source -> 77 us)
+  const long long ni = sel_items(items), wave = 3 * 152, share = (wave + ni - 1) / ni, four = (n + 4 * KB - 1) / (4 * KB);
+  long long gb = (n + KB - 1) / KB, most = share > four ? share : four;
+  if (gb > most) gb = most;
+  if (gb > wave) gb = wave;
   const dim3 g((unsigned)(gb < 1 ? 1 : gb), sel_items(items));
   float4* vj = V + (size_t)j * items * n;
   float4* vn = V + (size_t)(j + 1) * items * n;

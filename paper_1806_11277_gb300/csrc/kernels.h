@@ -277,7 +277,7 @@ void launch_cast_c64_c128(long long n, const float2* in, double2* out, cudaStrea
 void launch_copy(long long nbytes, const void* in, void* out, cudaStream_t s);
 // partial dot products: part[item][i][blk] = sum conj(V_i) w over block blk
 // V: [m+1][items][n] (vector i of item b at V + (i*items + b)*n)
-int krylov_nblk(long long n);
+int krylov_nblk(long long n, int items);
 void launch_mdot(long long n, int items, int nv, const double2* V, const double2* w, double2* part,
                  int nblk, cudaStream_t s);
 // w -= sum_i V_i h_i; if dot: partial dots of V with the new w; if nrm: partial |w|^2
