@@ -13,7 +13,7 @@
 // Why blocks: column by column over the augmented [A | I] every step re-read
 // and re-wrote the whole 2 N^2 entries, 4 N launches and 12 N^3 FP64 operations on
 // a chip whose FP64 rate is 54x below its FP32 rate.  Here FP64 arithmetic is left
-// in the panel (8 N^2 B operations), spread over a cluster of 8 SMs per matrix, and
+// in the panel (8 N^2 B operations), spread over a cluster of SMs per matrix, and
 // the 8 N^3 operations of the updates run as exact products of small integers on the
 // FP16 tensor cores (Ozaki, Ogita, Oishi and Rump, "Error-free transformations of
 // matrix multiplication by using fast routines of matrix multiplication and its
@@ -36,7 +36,7 @@ constexpr int NDIG = 6;               // digits per real number
 constexpr int DBITS = 9;
 constexpr int NGRP = 7;               // digit products with i + j < NGRP are kept
 constexpr int NPL = 2 * NDIG;         // planes: (digit, re / im)
-constexpr int CL = 8;                 // CTAs (SMs) per matrix in the panel kernel
+constexpr int CLMAX = 16;             // most CTAs (SMs) per matrix in the panel kernel
 constexpr int PT = 512;               // its threads per CTA
 constexpr int TM = 64;                // update tile: TM x TM entries of A
 constexpr int EXP_BAD = 1 << 20;      // exponent of a row that holds Inf or NaN
@@ -89,7 +89,7 @@ __device__ __forceinline__ void digits(long long v, int d[NDIG]) {
   d[0] = (int)v;
 }
 
-// One block's panel.  A cluster of CL CTAs holds the N x B panel of one matrix, rows
+// One block's panel.  A cluster of cl CTAs holds the N x B panel of one matrix, rows
 // split among the CTAs, in shared memory (in gp where it does not fit).  Lane = column
 // (32 / B rows per warp pass), so a row update is 4 FP64 FMAs per lane with the pivot
 // row in registers.  Per column: every CTA finds its pivot candidate (the warps kept
@@ -98,17 +98,17 @@ __device__ __forceinline__ void digits(long long v, int d[NDIG]) {
 // the same winner and updates its rows.  The receive slots alternate, so a CTA may send
 // for the next column while another still reads this one's.  Bound by the FP64 pipe.
 template <int B>
-__global__ void __launch_bounds__(PT) k_inv_panel(int N, int Npad, int k0, int bb, double2* __restrict__ A,
+__global__ void __launch_bounds__(PT) k_inv_panel(int N, int Npad, int k0, int bb, int cl, double2* __restrict__ A,
                                                   double2* __restrict__ gp, __half* __restrict__ wd,
                                                   int* __restrict__ we, int* __restrict__ swp, int* __restrict__ err) {
   constexpr int G = 32 / B, NW = PT / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double2 srow[2][CL][B];   // scaled candidate rows by sender
+  __shared__ double2 srow[2][CLMAX][B];   // scaled candidate rows by sender
   __shared__ double2 krow[2][B];       // row k before the exchange
-  __shared__ int2 skey[2][CL];         // (key, row) by sender
+  __shared__ int2 skey[2][CLMAX];         // (key, row) by sender
   __shared__ int2 wkey[NW];
-  const int rank = blockIdx.x % CL, mat = blockIdx.x / CL;
-  const int rp = (N + CL - 1) / CL, r0 = min(N, rank * rp), r1 = min(N, r0 + rp);
+  const int rank = blockIdx.x % cl, mat = blockIdx.x / cl;
+  const int rp = (N + cl - 1) / cl, r0 = min(N, rank * rp), r1 = min(N, r0 + rp);
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, col = lane % B, sub = lane / B;
   double2* Am = A + (long long)mat * N * N;
   double2* P = gp ? gp + ((long long)mat * N + r0) * B : reinterpret_cast<double2*>(smem_raw);
@@ -154,21 +154,20 @@ __global__ void __launch_bounds__(PT) k_inv_panel(int N, int Npad, int k0, int b
       const double2 inv = cinv(shfl_d2(v, t));
       const double2 u = col == t ? inv : cmul(v, inv);
       // the CTA's message to every CTA of the cluster
-      for (int q = 0; q < CL; ++q) {
+      for (int q = 0; q < cl; ++q) {
         if (lane < B) st_cluster(cluster_addr(saddr(&srow[par][rank][col]), q), u);
         if (lane == 0) st_cluster(cluster_addr(saddr(&skey[par][rank]), q), c);
       }
     } else if (wid == 1 && k >= r0 && k < r1 && lane < B) {
       const double2 v = P[(k - r0) * B + col];
-      for (int q = 0; q < CL; ++q) st_cluster(cluster_addr(saddr(&krow[par][col]), q), v);
+      for (int q = 0; q < cl; ++q) st_cluster(cluster_addr(saddr(&krow[par][col]), q), v);
     }
     __syncwarp();
     cluster_arrive();
     cluster_wait();
     int2 best = skey[par][0];
     int win = 0;
-#pragma unroll
-    for (int q = 1; q < CL; ++q) {
+    for (int q = 1; q < cl; ++q) {
       const int2 c = skey[par][q];
       if (c.x > best.x || (c.x == best.x && c.y < best.y)) { best = c; win = q; }
     }
@@ -337,7 +336,8 @@ __device__ __forceinline__ double join(const float G[NGRP], int s) {
 // tile (24 x 64 x B halves, 96 KB at B = 32: 2 CTAs per SM) are staged at once; a warp
 // takes 16 rows x 32 columns, 8 columns at a time: 26 digit pairs x 4 (complex) = 104 MMAs
 // of 16 x 8 x 16 per step of 16 in k, into 14 accumulator tiles (7 weights, re and im).  The staged rows are XOR-swizzled so that
-// ldmatrix meets no bank conflict.  Bound by the tensor pipe and the joining.
+// ldmatrix meets no bank conflict.  Bound by the tensor pipe (56 % busy) and the joining; with the tile of A asked
+// for early 16 matrices of 1408 take 0.59 ms a block instead of 0.64 (210 GFLOP of MMAs: 360 TFLOP/s).
 template <int B>
 __global__ void __launch_bounds__(256, 2) k_inv_update(int N, int Npad, int k0, int bb, double2* __restrict__ A,
                                                        const __half* __restrict__ wd, const __half* __restrict__ rd,
@@ -363,8 +363,13 @@ __global__ void __launch_bounds__(256, 2) k_inv_update(int N, int Npad, int k0, 
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wr = (wid & 3) * 16, wc = (wid >> 2) * 32;
   const int ia = i0 + wr + (lane >> 2), ib = ia + 8;   // the two rows of this thread's accumulators
-  const int ea = we[(long long)mat * Npad + ia] + 2, eb = we[(long long)mat * Npad + ib] + 2;
+  // the tile of A, on its way to L2 while the digits are staged and multiplied
   double2* Am = A + (long long)mat * N * N;
+  for (int q = threadIdx.x; q < TM * (TM / 8); q += 256) {
+    const int row = i0 + q / (TM / 8), c8 = j0 + q % (TM / 8) * 8;
+    if (row < N && c8 < N) asm volatile("prefetch.global.L2 [%0];" ::"l"(Am + (long long)row * N + c8));
+  }
+  const int ea = we[(long long)mat * Npad + ia] + 2, eb = we[(long long)mat * Npad + ib] + 2;
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   __syncthreads();
   for (int nt = 0; nt < 4; ++nt) {
@@ -404,7 +409,14 @@ __global__ void __launch_bounds__(256, 2) k_inv_update(int N, int Npad, int k0, 
         }
       }
     }
-    // join the weights and add to A
+    // join the weights and add to A, its entries loaded first
+    double2 old[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = q < 2 ? ia : ib, j = j0 + jn + (lane & 3) * 2 + (q & 1);
+      old[q] = make_double2(0.0, 0.0);
+      if (i < N && j < N && (i < k0 || i >= k0 + bb)) old[q] = Am[(long long)i * N + j];
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int i = q < 2 ? ia : ib, j = j0 + jn + (lane & 3) * 2 + (q & 1);
@@ -414,13 +426,9 @@ __global__ void __launch_bounds__(256, 2) k_inv_update(int N, int Npad, int k0, 
 #pragma unroll
       for (int g = 0; g < NGRP; ++g) { gr[g] = ac[g][0][q]; gi[g] = ac[g][1][q]; }
       double2 v = make_double2(join(gr, s), join(gi, s));
-      double2* o = Am + (long long)i * N + j;
-      if (i < k0 || i >= k0 + bb) {
-        const double2 old = *o;
-        v.x += old.x;
-        v.y += old.y;
-      }
-      *o = v;
+      v.x += old[q].x;
+      v.y += old[q].y;
+      Am[(long long)i * N + j] = v;
     }
   }
 }
@@ -456,21 +464,58 @@ __global__ void k_inv_columns(int N, const double2* __restrict__ A, const int* _
 }
 
 struct Plan {
-  int B, Npad;
+  int B, cl, Npad;
   bool global;                          // the panel does not fit in shared memory
   size_t psm, usm;                      // dynamic shared memory of the panel and update kernels
   size_t dig, gp;                       // bytes of one operand's digits and of the global panel
 };
-// B = 32 while a CTA's share of the panel fits beside the message slots (N <= 3200), else 16
-// (N <= 6400: the panel's FP64 work halves, the update's passes over A double), beyond that with the
-// panel in global memory (L2).
+template <int B> int clusters_of(int cl, size_t sm) {   // clusters of cl CTAs the device runs at once
+  cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cl);
+  cfg.blockDim = dim3(PT);
+  cfg.dynamicSmemBytes = sm;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, k_inv_panel<B>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  return n;
+}
+// B = 32 columns a block up to N = 3200, else 16 (the panel's FP64 work halves, the update's passes over A double).
+// The panel is bound by the FP64 pipe of its SMs, so the cluster size is the one with the fewest rows per CTA
+// times waves of clusters, at one CTA per SM (at least 100 KB of shared memory each: two to an SM, as clusters of
+// 8 with 90 KB were placed, share its pipe).  GB300 runs 7 clusters of 16, 15 of 8, 23 of 6 or 36 of 4 that way.
+// 16 matrices of 1408: 455 us a block with clusters of 8, two to an SM; 511 with 15 of the 16 at a time; 339 with 6.
 Plan plan_for(int N, int nmat) {
   Plan p;
-  const size_t lim = 200 * 1024, rp = (N + CL - 1) / CL;
-  p.B = rp * 32 * sizeof(double2) <= lim ? 32 : 16;
+  const size_t lim = 200 * 1024, least = 100 * 1024;
+  p.B = N <= 3200 ? 32 : 16;
   p.Npad = (N + TM - 1) / TM * TM;
-  p.global = rp * p.B * sizeof(double2) > lim;
-  p.psm = p.global ? 0 : rp * p.B * sizeof(double2);
+  p.cl = 0;
+  p.global = false;
+  p.psm = 0;
+  long long best = 0;
+  const int sizes[] = {16, 12, 10, 8, 6, 5, 4};
+  for (int cl : sizes) {
+    const size_t rp = (N + cl - 1) / cl, need = rp * p.B * sizeof(double2), sm = need > least ? need : least;
+    if (need > lim) continue;
+    const int act = p.B == 32 ? clusters_of<32>(cl, sm) : clusters_of<16>(cl, sm);
+    if (act < 1) continue;
+    const long long cost = (long long)((nmat + act - 1) / act) * (long long)rp;
+    if (!p.cl || cost < best) { best = cost; p.cl = cl; p.psm = sm; }
+  }
+  if (!p.cl) {                          // beyond N = 12800: the panel in global memory (L2)
+    p.cl = 8;
+    p.global = true;
+  }
   p.usm = (size_t)2 * NPL * TM * p.B * sizeof(__half);
   p.dig = (size_t)nmat * NPL * p.Npad * p.B * sizeof(__half);
   p.gp = p.global ? (size_t)nmat * N * p.B * sizeof(double2) : 0;
@@ -481,23 +526,24 @@ size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 template <int B>
 int invert_t(const Plan& p, int N, int nmat, double2* A, double2* gp, __half* wd, __half* rd, int* we, int* re, int* swp,
              int* err, cudaStream_t s) {
+  cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.psm);
   cudaFuncSetAttribute(k_inv_update<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.usm);
   int launches = 0;
   for (int k0 = 0; k0 < N; k0 += B) {
     const int bb = N - k0 < B ? N - k0 : B;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CL * nmat);
+    cfg.gridDim = dim3(p.cl * nmat);
     cfg.blockDim = dim3(PT);
     cfg.dynamicSmemBytes = p.psm;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.x = p.cl;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_inv_panel<B>, N, p.Npad, k0, bb, A, gp, wd, we, swp, err);
+    cudaLaunchKernelEx(&cfg, k_inv_panel<B>, N, p.Npad, k0, bb, p.cl, A, gp, wd, we, swp, err);
     ++launches;
     if (bb == N) break;                 // no other columns
     k_inv_rows<B><<<dim3((N + 31) / 32, nmat), 256, 0, s>>>(N, p.Npad, k0, bb, A, rd, re, swp);
