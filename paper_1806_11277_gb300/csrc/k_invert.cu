@@ -469,9 +469,15 @@ struct Plan {
   size_t psm, usm;                      // dynamic shared memory of the panel and update kernels
   size_t dig, gp;                       // bytes of one operand's digits and of the global panel
 };
-template <int B> int clusters_of(int cl, size_t sm) {   // clusters of cl CTAs the device runs at once
+// Function attributes are the process's, so they are always set to the same values (threads may build contexts side
+// by side).
+constexpr int PANEL_SMEM = 200 * 1024, PERM_SMEM = 2 * 16384 * (int)sizeof(int);
+template <int B> void panel_attributes() {
   cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM);
+}
+template <int B> int clusters_of(int cl, size_t sm) {   // clusters of cl CTAs the device runs at once
+  panel_attributes<B>();
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cl);
   cfg.blockDim = dim3(PT);
@@ -496,7 +502,7 @@ template <int B> int clusters_of(int cl, size_t sm) {   // clusters of cl CTAs t
 // 16 matrices of 1408: 455 us a block with clusters of 8, two to an SM; 511 with 15 of the 16 at a time; 339 with 6.
 Plan plan_for(int N, int nmat) {
   Plan p;
-  const size_t lim = 200 * 1024, least = 100 * 1024;
+  const size_t lim = PANEL_SMEM, least = 100 * 1024;
   p.B = N <= 3200 ? 32 : 16;
   p.Npad = (N + TM - 1) / TM * TM;
   p.cl = 0;
@@ -526,8 +532,7 @@ size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 template <int B>
 int invert_t(const Plan& p, int N, int nmat, double2* A, double2* gp, __half* wd, __half* rd, int* we, int* re, int* swp,
              int* err, cudaStream_t s) {
-  cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  cudaFuncSetAttribute(k_inv_panel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.psm);
+  panel_attributes<B>();
   cudaFuncSetAttribute(k_inv_update<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.usm);
   int launches = 0;
   for (int k0 = 0; k0 < N; k0 += B) {
@@ -574,7 +579,7 @@ int dense_invert(int N, int nmat, double2* A, double2* inv, void* ws, int* err, 
   cudaMemsetAsync(ws, 0, dense_invert_workspace(N, nmat), s);
   int n = p.B == 32 ? invert_t<32>(p, N, nmat, A, gp, wd, rd, we, re, swp, err, s)
                     : invert_t<16>(p, N, nmat, A, gp, wd, rd, we, re, swp, err, s);
-  cudaFuncSetAttribute(k_inv_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * N * sizeof(int)));
+  cudaFuncSetAttribute(k_inv_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, PERM_SMEM);
   k_inv_perm<<<nmat, 256, 2 * N * sizeof(int), s>>>(N, swp, perm);
   k_inv_columns<<<dim3((N + 255) / 256, N, nmat), 256, 0, s>>>(N, A, perm, inv);
   return n + 2;
