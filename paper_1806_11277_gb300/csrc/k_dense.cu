@@ -194,8 +194,8 @@ __global__ void __launch_bounds__(256) k_dense_apply_vs(int N, int nrhs, int nsu
   pdl_trigger();
   const int row0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4;
   if (row0 < N) {
-    // il may be from the launch before this one and not yet written: then it holds older items, and what is
-    // asked for early is of no use, no more
+    // il may be from the launch before this one and not yet written: then it holds older items of the batch (zeros
+    // from setup at first), and what is asked for early is of no use, no more
     const int early = il ? il[blockIdx.y] : blockIdx.y;
     prefetch_rows(inv + ((long long)(early / nrhs) * N + row0) * N, (long long)N * sizeof(TI), 4, pre);
   }

@@ -366,30 +366,29 @@ __global__ void __launch_bounds__(128) k_st_vupd_full(Grid g, int nrhs, const TI
   }
 }
 
-// MG-DD colour residual fused with its gather: local unknown e of sub-item bl
+// MG-DD colour residual fused with its gather (2D): local unknown e of sub-item bl
 // (= ((m * nsub) + s) * nrhs + r) receives (b - K_c x) at coarsest slot
 // map[s][e] of item m * nrhs + r, or 0 on padding (map -1); only the rows of
-// the colour's subdomains are evaluated.  Two warps share 32 rows, each summing
-// the coefficients of one slot parity (a warp-uniform split: no divergence),
-// so that twice as many loads are in flight (the launch is small: the box
-// unknowns of one colour); the halves meet in shared memory.
-template <typename T, typename TT, int D, int LV, bool SYM>
-__device__ __forceinline__ typename CT<T>::type gather_row_half(const Grid& g, const TT* ts, long long c,
-                                                                const int i[3], const typename CT<T>::type* x,
-                                                                int a, int part) {
-  if (part == 0) {
-    if (a == 0) return st_row_ct<T, TT, D, LV, SYM, 0, false, 2, 0>(g, ts, c, i, x);
-    if (a == 1) return st_row_ct<T, TT, D, LV, SYM, 1, false, 2, 0>(g, ts, c, i, x);
-    if (a == 2) return st_row_ct<T, TT, D, LV, SYM, 2, false, 2, 0>(g, ts, c, i, x);
+// the colour's subdomains are evaluated.  The launch is small (the box unknowns of one
+// colour) and bound by latency, so NS warps share 32 rows, each summing the
+// coefficients of one residue of the slot modulo NS (a warp-uniform split: no
+// divergence); the shares meet in shared memory.
+template <typename T, typename TT, int LV, bool SYM, int NS, int SI = 0>
+__device__ __forceinline__ typename CT<T>::type gather_share(const Grid& g, const TT* ts, long long c, const int i[3],
+                                                             const typename CT<T>::type* x, int a, int part) {
+  if constexpr (SI < NS) {
+    if (part == SI) {
+      if (a == 0) return st_row_ct<T, TT, 2, LV, SYM, 0, false, NS, SI>(g, ts, c, i, x);
+      if (a == 1) return st_row_ct<T, TT, 2, LV, SYM, 1, false, NS, SI>(g, ts, c, i, x);
+      if (a == 2) return st_row_ct<T, TT, 2, LV, SYM, 2, false, NS, SI>(g, ts, c, i, x);
+    }
+    return gather_share<T, TT, LV, SYM, NS, SI + 1>(g, ts, c, i, x, a, part);
   } else {
-    if (a == 0) return st_row_ct<T, TT, D, LV, SYM, 0, false, 2, 1>(g, ts, c, i, x);
-    if (a == 1) return st_row_ct<T, TT, D, LV, SYM, 1, false, 2, 1>(g, ts, c, i, x);
-    if (a == 2) return st_row_ct<T, TT, D, LV, SYM, 2, false, 2, 1>(g, ts, c, i, x);
+    return czero<typename CT<T>::type>();
   }
-  return czero<typename CT<T>::type>();
 }
 
-template <typename T, typename TT, int D, int LV, bool SYM>
+template <typename T, typename TT, int LV, bool SYM, int NS>
 __global__ void __launch_bounds__(128) k_st_resid_gather(Grid g, int nrhs, int nsub, int nloc,
                                                          const int* __restrict__ map, const TT* __restrict__ tab,
                                                          const typename CT<T>::type* x,
@@ -398,31 +397,31 @@ __global__ void __launch_bounds__(128) k_st_resid_gather(Grid g, int nrhs, int n
                                                          const int* il) {
   pdl_enter();
   typedef typename CT<T>::type Cx;
-  constexpr StencilLayout L = level_layout(D, LV);
-  __shared__ Cx half1[2][32];
+  constexpr StencilLayout L = level_layout(2, LV);
+  constexpr int RG = 4 / NS;
+  __shared__ Cx sp[NS - 1][RG][32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int part = w & 1;                                  // slot parity this warp sums
-  const int e = blockIdx.x * 64 + (w >> 1) * 32 + lane;
+  const int part = w % NS, rg = w / NS;                    // residue of the slots this warp sums
+  const int e = blockIdx.x * (32 * RG) + rg * 32 + lane;
   const int bl = il ? il[blockIdx.y] : blockIdx.y;
   const int r = bl % nrhs, s = (bl / nrhs) % nsub, m = bl / (nrhs * nsub);
   const long long N = g.ncell;
   const int gs = e < nloc ? map[(long long)s * nloc + e] : -1;
   Cx v = czero<Cx>();
-  const long long vo = (long long)(m * nrhs + r) * (D + 1) * N;
+  const long long vo = (long long)(m * nrhs + r) * 3 * N;
   if (gs >= 0) {
     const int a = gs / (int)N, c = gs - a * (int)N;
-    constexpr int nslot = SYM ? half_base(L, L.npair) : L.nslot;
-    const TT* ts = tab + (long long)m * nslot * N;
     int i[3];
     cell_coords(g, c, i);
-    v = gather_row_half<T, TT, D, LV, SYM>(g, ts, c, i, x + vo, a, part);
+    constexpr int nslot = SYM ? half_base(L, L.npair) : L.nslot;
+    const TT* ts = tab + (long long)m * nslot * N;
+    v = gather_share<T, TT, LV, SYM, NS>(g, ts, c, i, x + vo, a, part);
   }
-  if (part) half1[w >> 1][lane] = v;
+  if (part) sp[part - 1][rg][lane] = v;
   __syncthreads();
   if (!part && e < nloc) {
-    const Cx v1 = half1[w >> 1][lane];
-    v.x += v1.x;
-    v.y += v1.y;
+#pragma unroll
+    for (int q = 1; q < NS; ++q) v = cadd(v, sp[q - 1][rg][lane]);
     if (gs >= 0) v = csub(*(b + vo + gs), v);
     out[(long long)bl * nloc + e] = v;
   }
@@ -553,13 +552,28 @@ __global__ void k_table_half(long long n, const double2* __restrict__ in, void* 
   if (fmt == 1) ((__half2*)out)[i] = __floats2half2_rn((float)v.x, (float)v.y);
   else ((__nv_bfloat162*)out)[i] = __floats2bfloat162_rn((float)v.x, (float)v.y);
 }
+// NS = 4 up to 200 K unknowns in all boxes of the batch (with every item active: the order of the sums does not change
+// while items converge), 2 above.  A 512^2 MG-DD cycle of one medium (90 K unknowns in four colours): 233.8 us with 2,
+// 223.5 with 4; of two media 348 and 346; of four 582 and 592.
+template <typename T, typename TT, bool SYM, int NS>
+static void resid_gather_n(const Grid& g, int items_l, int nrhs, int nsub, int nloc, const int* map, int v,
+                           const TT* tab, const typename CT<T>::type* x, const typename CT<T>::type* b,
+                           typename CT<T>::type* out, cudaStream_t s) {
+  constexpr int per = 128 / NS;            // unknowns per 128-thread block
+  const dim3 gr((unsigned)((nloc + per - 1) / per), sel_items(items_l));
+  if (v == 1)
+    launch_pdl(gr, 128, 0, s, k_st_resid_gather<T, TT, 1, SYM, NS>, g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
+  else
+    launch_pdl(gr, 128, 0, s, k_st_resid_gather<T, TT, 2, SYM, NS>, g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
+}
 template <typename T, typename TT, bool SYM>
 static void resid_gather_t(const Grid& g, int items_l, int nrhs, int nsub, int nloc, const int* map, int v,
                            const TT* tab, const typename CT<T>::type* x, const typename CT<T>::type* b,
                            typename CT<T>::type* out, cudaStream_t s) {
-  const dim3 gr((unsigned)((nloc + 63) / 64), sel_items(items_l));   // 64 unknowns per 128-thread block
-  if (v == 1) launch_pdl(gr, 128, 0, s, k_st_resid_gather<T, TT, 2, 1, SYM>, g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
-  else launch_pdl(gr, 128, 0, s, k_st_resid_gather<T, TT, 2, 2, SYM>, g, nrhs, nsub, nloc, map, tab, x, b, out, g_sel.list);
+  if ((long long)nloc * items_l <= 200000)
+    resid_gather_n<T, TT, SYM, 4>(g, items_l, nrhs, nsub, nloc, map, v, tab, x, b, out, s);
+  else
+    resid_gather_n<T, TT, SYM, 2>(g, items_l, nrhs, nsub, nloc, map, v, tab, x, b, out, s);
 }
 
 template <typename T>

@@ -51,3 +51,24 @@ def test_split_rows_equal_whole_rows(shape, levels, media, nrhs, half, monkeypat
     for a, b in zip(*got):
         tol = 2e-5 if a.dtype == torch.complex64 else 1e-12
         assert float((a - b).abs().max() / b.abs().max()) <= tol
+
+
+# MG-DD colour residuals: a row over two warps above 200 K box unknowns, over four below (a right-hand side alone);
+# boxes whose unknowns end inside a block, and unequal ones
+@pytest.mark.parametrize("shape,split", [((128, 160), (4, 4, 1)), ((160, 152), (4, 3, 1))])
+@pytest.mark.parametrize("fmt", [0, 2])
+def test_gather_of_a_large_batch_equals_single_ones(shape, split, fmt):
+    n = 32
+    med = [synth.random_2d(n=shape[0], nx=shape[1], sigma=0.3, seed=7, corr=4.0, abl=2)]
+    kw = dict(levels=3, alpha=0.4, coarse_dd=split, coarse_dd_overlap=3, coarse_fmt=fmt, coef_half=1 if fmt else 0)
+    with ehs.solver_for(med, nrhs=n, **kw) as S, ehs.solver_for(med, nrhs=1, **kw) as S1:
+        for dt in (torch.complex64, torch.complex128):
+            b = _vec(S.level_shape(0), dt, 3)
+            x = torch.empty_like(b)
+            S.vcycle(b, x)
+            # twice the bar of one cycle against the FP64 oracle
+            tol = 1e-4 if dt == torch.complex64 else 2e-10
+            for i in (0, n - 1):
+                x1 = torch.empty_like(b[i:i + 1])
+                S1.vcycle(b[i:i + 1].contiguous(), x1)
+                assert float((x[i] - x1[0]).abs().max() / x1.abs().max()) <= tol
