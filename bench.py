@@ -79,7 +79,7 @@ ROOF_KERNEL = ("k_dense_apply_vs<__half2> (MG-DD coarsest local products with th
 ST_ROWS_L1_BYTES_PER_CELL = 45 * 4 + 24 + 24
 # DRAM read + write bytes of one roofline-kernel launch (one colour) of the default line, from an
 # ncu capture of the kernel as it stands (None whenever the kernel changes): mean of 7 warm launches
-ROOF_TRAFFIC_C2 = 447.13e6 + 0.59e6
+ROOF_TRAFFIC_C2 = 451.34e6 + 0.59e6
 
 # Stencil kernels of the default line (the metric's "stencil HBM GB/s"), each timed through the
 # C ABI call that launches it alone: algorithmic bytes per cell of the level it runs on (each
