@@ -402,13 +402,16 @@ void build_hier(ehs_ctx* c, Hier& H, int precs, bool coef_only) {
   const long long N = nloc;
   double2* M = dalloc<double2>(c, (size_t)nmat * N * N);
   unsigned char* iws = dalloc<unsigned char>(c, dense_invert_workspace((int)N, nmat));
+  int* ex = dalloc<int>(c, (size_t)H.nsets * NG);               // equilibration of the coarsest unknowns
+  int* exl = mgdd ? dalloc<int>(c, (size_t)nmat * N) : ex;      // and of the matrices' rows
+  launch_dense_scale(C.g, H.nsets, C.L, C.tab64, ex, c->s); cnt(2);
   if (mgdd)
-    launch_dense_assemble_sub(C.g, H.nsets, H.cdd.nsub, nloc, C.L, C.tab64, H.cdd.d_map, d_g2l, M, c->s);
+    launch_dense_assemble_sub(C.g, H.nsets, H.cdd.nsub, nloc, C.L, C.tab64, ex, H.cdd.d_map, d_g2l, M, exl, c->s);
   else
-    launch_dense_assemble(C.g, H.nsets, C.L, C.tab64, M, c->s);
+    launch_dense_assemble(C.g, H.nsets, C.L, C.tab64, ex, M, c->s);
   cnt(); post();
   C.inv = dalloc<double2>(c, (size_t)nmat * N * N);
-  cnt(dense_invert((int)N, nmat, M, C.inv, iws, derr, c->s)); post();
+  cnt(dense_invert((int)N, nmat, M, exl, C.inv, iws, derr, c->s)); post();
   if (precs & 2) {
     if (H.coarse_fmt == 1) {
       C.invlp = dalloc<float2>(c, (size_t)nmat * N * N);
@@ -424,7 +427,8 @@ void build_hier(ehs_ctx* c, Hier& H, int precs, bool coef_only) {
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, c->s));
   CK(cudaStreamSynchronize(c->s));
-  dfree(c, M); dfree(c, iws); dfree(c, derr);
+  dfree(c, M); dfree(c, iws); dfree(c, derr); dfree(c, ex);
+  if (mgdd) dfree(c, exl);
   if (d_g2l) dfree(c, d_g2l);
   if (!(precs & 1)) { dfree(c, C.inv); C.inv = nullptr; }
   if (herr & EHS_DEVERR_BOX) throw CudaError("Galerkin stencil fell outside its box");

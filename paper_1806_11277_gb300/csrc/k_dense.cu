@@ -4,6 +4,13 @@
 // coarsest LU does).  Boundary slots are identity rows so the dense index is
 // simply comp * ncell + cell.
 //
+// The matrices are assembled equilibrated, D A D with D a diagonal of powers of two (k_dense_scale), and the
+// inverse is scaled back by D from both sides (k_invert.cu): exact scalings, and what is inverted no longer depends
+// on the units of the medium.  Displacements and pressures differ in scale by sqrt(mu (lambda + mu)) / h, near 1
+// in km, km/s and g/cm^3 with h = 1 and about 2^30 in SI units with h = 10 m, and the inverse's digits hold the entries of a
+// row to 2^-55 of the largest: without D the inverse of an SI medium (12 x 14 coarsest cells) is off by 2.5e-8, with
+// it by 1.2e-15 (numpy restatement; FP64 elimination column by column 2.5e-15 in either units).
+//
 // MG-DD (Sec. 4): the same machinery for the subdomains of the coarsest grid.
 // Each box's local matrix (the coarsest operator restricted to the box
 // unknowns, padded with identity rows to nloc) is assembled from the stencil
@@ -16,14 +23,71 @@
 namespace ehs {
 namespace {
 
+// x 2^e
+__device__ __forceinline__ double2 scaled(double2 v, int e) { return make_double2(ldexp(v.x, e), ldexp(v.y, e)); }
+// floor(log2 of the larger part), NONE for zero (and what is below the normal range)
+constexpr int NONE = -8192;
+__device__ __forceinline__ int exponent(double2 v) {
+  const int h = max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) >> 20;
+  return h ? h - 1023 : NONE;
+}
+
+// Exponents ex of the equilibration D (d = 2^ex) of the coarsest unknowns, [nsets][(D + 1) ncell].  Displacements
+// (pass 0): the largest entry of the row towards its own component, of size about one after scaling (the diagonal
+// alone may cancel between stiffness and mass).  Pressures (pass 1): half of the same, so that pivots stay on the
+// diagonal (error of the inverse in km units 1.1e-15, 2.9e-15 without that half), but no larger than what leaves the
+// largest coupling to a scaled displacement in [2, 4): a nearly incompressible medium, whose pressure diagonal is
+// tiny, keeps its displacement block (lambda / mu = 1e6: 2.4e-15, 6.9e-14 from the diagonal alone, and a pressure block
+// ten times worse with the coupling in [1/2, 1)).  A thread per row, once per context.
 template <int D>
-__global__ void k_dense_assemble(Grid g, StencilLayout L, const double2* __restrict__ tab,
+__global__ void k_dense_scale(Grid g, StencilLayout L, const double2* __restrict__ tab, int* ex, int pass) {
+  const long long N = (long long)(D + 1) * g.ncell;
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= N) return;
+  const int a = (int)(r / g.ncell);
+  if ((a == D) != (pass == 1)) return;
+  const double2* ts = tab + (long long)blockIdx.y * L.nslot * g.ncell;
+  int* es = ex + (long long)blockIdx.y * N;
+  const long long c = r % g.ncell;
+  int i[3];
+  cell_coords(g, c, i);
+  if (!slot_valid(a, D, i)) { es[r] = 0; return; }
+  int own = NONE, coup = NONE;
+  for (int q = L.row_first[a]; q < L.row_first[a + 1]; ++q) {
+    const PairBox& P = L.p[q];
+    if (P.b != a && a != D) continue;
+    int s = P.base;
+    for (int oz = 0; oz < P.ext[2]; ++oz)
+      for (int oy = 0; oy < P.ext[1]; ++oy)
+        for (int ox = 0; ox < P.ext[0]; ++ox, ++s) {
+          const int j[3] = {i[0] + P.lo[0] + ox, i[1] + P.lo[1] + oy, i[2] + P.lo[2] + oz};
+          bool in = true;
+          for (int k = 0; k < 3; ++k) in = in && j[k] >= 0 && j[k] < g.n[k];
+          if (!in || !slot_valid(P.b, D, j)) continue;
+          const int e = exponent(ts[(long long)s * g.ncell + c]);
+          if (e == NONE) continue;
+          if (P.b == a) own = max(own, e);
+          else coup = max(coup, e + es[(long long)P.b * g.ncell + cell_index(g, j)]);
+        }
+  }
+  int e = own == NONE ? 0 : -((own + 1) >> 1);
+  if (a == D) {
+    e -= 1;
+    if (coup != NONE) e = own == NONE ? 1 - coup : min(e, 1 - coup);
+  }
+  es[r] = e;
+}
+
+// A: D K_c D, zeroed before
+template <int D>
+__global__ void k_dense_assemble(Grid g, StencilLayout L, const double2* __restrict__ tab, const int* __restrict__ ex,
                                  double2* __restrict__ A) {
   const long long N = (long long)(D + 1) * g.ncell;
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= N) return;
   const int set = blockIdx.y;
   const double2* ts = tab + (long long)set * L.nslot * g.ncell;
+  const int* es = ex + (long long)set * N;
   double2* row = A + ((long long)set * N + r) * N;
   const int a = (int)(r / g.ncell);
   const long long c = r % g.ncell;
@@ -40,8 +104,8 @@ __global__ void k_dense_assemble(Grid g, StencilLayout L, const double2* __restr
           bool in = true;
           for (int k = 0; k < 3; ++k) in = in && j[k] >= 0 && j[k] < g.n[k];
           if (!in || !slot_valid(P.b, D, j)) continue;
-          const double2 v = ts[(long long)s * g.ncell + c];
           const long long col = (long long)P.b * g.ncell + cell_index(g, j);
+          const double2 v = scaled(ts[(long long)s * g.ncell + c], es[r] + es[col]);
           row[col].x += v.x;
           row[col].y += v.y;
         }
@@ -81,11 +145,12 @@ __global__ void k_dense_apply(int N, int nrhs, const double2* __restrict__ inv,
 // MG-DD local problems (Sec. 4): row e of local matrix (set, s) is the
 // coarsest-level row of global slot map[s][e], restricted to the columns that
 // are local unknowns of subdomain s (g2l[s][slot] >= 0); padding rows (map -1)
-// are identity rows.  A comes zeroed, as for k_dense_assemble.
+// are identity rows.  A comes zeroed and goes out equilibrated, as for k_dense_assemble; exl: the
+// exponents of its rows.
 template <int D>
-__global__ void k_dense_assemble_sub(Grid g, StencilLayout L, const double2* __restrict__ tab, int nsub,
-                                     int nloc, const int* __restrict__ map, const int* __restrict__ g2l,
-                                     double2* __restrict__ A) {
+__global__ void k_dense_assemble_sub(Grid g, StencilLayout L, const double2* __restrict__ tab,
+                                     const int* __restrict__ ex, int nsub, int nloc, const int* __restrict__ map,
+                                     const int* __restrict__ g2l, double2* __restrict__ A, int* __restrict__ exl) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nloc) return;
   const int ms = blockIdx.y;                 // set * nsub + s
@@ -94,7 +159,9 @@ __global__ void k_dense_assemble_sub(Grid g, StencilLayout L, const double2* __r
   const double2* ts = tab + (long long)set * L.nslot * g.ncell;
   double2* row = A + ((long long)ms * nloc + e) * nloc;
   const int gs = map[(long long)sub * nloc + e];
-  if (gs < 0) { row[e] = make_double2(1, 0); return; }
+  if (gs < 0) { row[e] = make_double2(1, 0); exl[(long long)ms * nloc + e] = 0; return; }
+  const int* es = ex + (long long)set * NG;
+  exl[(long long)ms * nloc + e] = es[gs];
   const int* gl = g2l + (long long)sub * NG;
   const int a = (int)(gs / g.ncell);
   const long long c = gs % g.ncell;
@@ -110,9 +177,10 @@ __global__ void k_dense_assemble_sub(Grid g, StencilLayout L, const double2* __r
           bool in = true;
           for (int k = 0; k < 3; ++k) in = in && j[k] >= 0 && j[k] < g.n[k];
           if (!in || !slot_valid(P.b, D, j)) continue;
-          const int lc = gl[(long long)P.b * g.ncell + cell_index(g, j)];
+          const long long gc = (long long)P.b * g.ncell + cell_index(g, j);
+          const int lc = gl[gc];
           if (lc < 0) continue;
-          const double2 v = ts[(long long)sl * g.ncell + c];
+          const double2 v = scaled(ts[(long long)sl * g.ncell + c], es[gs] + es[gc]);
           row[lc].x += v.x;
           row[lc].y += v.y;
         }
@@ -231,12 +299,22 @@ bool launch_dense_apply_scatter(int N, int items, int nrhs, int nsub, const int*
   return true;
 }
 
-void launch_dense_assemble(const Grid& g, int nsets, const StencilLayout& L, const double2* tab,
+void launch_dense_scale(const Grid& g, int nsets, const StencilLayout& L, const double2* tab, int* ex,
+                        cudaStream_t s) {
+  const long long N = (long long)(g.d + 1) * g.ncell;
+  dim3 grid((unsigned)((N + 127) / 128), nsets);
+  for (int pass = 0; pass < 2; ++pass) {
+    if (g.d == 2) k_dense_scale<2><<<grid, 128, 0, s>>>(g, L, tab, ex, pass);
+    else k_dense_scale<3><<<grid, 128, 0, s>>>(g, L, tab, ex, pass);
+  }
+}
+
+void launch_dense_assemble(const Grid& g, int nsets, const StencilLayout& L, const double2* tab, const int* ex,
                            double2* A, cudaStream_t s) {
   const long long N = (long long)(g.d + 1) * g.ncell;
   dim3 grid((unsigned)((N + 127) / 128), nsets);
-  if (g.d == 2) k_dense_assemble<2><<<grid, 128, 0, s>>>(g, L, tab, A);
-  else k_dense_assemble<3><<<grid, 128, 0, s>>>(g, L, tab, A);
+  if (g.d == 2) k_dense_assemble<2><<<grid, 128, 0, s>>>(g, L, tab, ex, A);
+  else k_dense_assemble<3><<<grid, 128, 0, s>>>(g, L, tab, ex, A);
 }
 
 template <typename T>
@@ -248,10 +326,11 @@ void launch_dense_apply(int N, int items, int nrhs, const double2* inv, const ty
 }
 
 void launch_dense_assemble_sub(const Grid& g, int nsets, int nsub, int nloc, const StencilLayout& L,
-                               const double2* tab, const int* map, const int* g2l, double2* A, cudaStream_t s) {
+                               const double2* tab, const int* ex, const int* map, const int* g2l, double2* A,
+                               int* exl, cudaStream_t s) {
   const dim3 grid((unsigned)((nloc + 127) / 128), nsets * nsub);
-  if (g.d == 2) k_dense_assemble_sub<2><<<grid, 128, 0, s>>>(g, L, tab, nsub, nloc, map, g2l, A);
-  else k_dense_assemble_sub<3><<<grid, 128, 0, s>>>(g, L, tab, nsub, nloc, map, g2l, A);
+  if (g.d == 2) k_dense_assemble_sub<2><<<grid, 128, 0, s>>>(g, L, tab, ex, nsub, nloc, map, g2l, A, exl);
+  else k_dense_assemble_sub<3><<<grid, 128, 0, s>>>(g, L, tab, ex, nsub, nloc, map, g2l, A, exl);
 }
 
 void launch_dense_apply_lp(int N, int items, int nrhs, int nsub, const int* sizes, const void* inv, int fmt,

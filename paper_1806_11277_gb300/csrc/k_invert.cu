@@ -25,6 +25,9 @@
 // matrices the inverse's error against an 80-bit one is about half that of the
 // FP64 column-by-column elimination (numpy restatement, N = 645: 4.0e-15 against
 // 7.7e-15 in the 2-norm); with the sums of i + j <= 5 only it would be five times larger.
+// An entry far below the largest of its row of W or column of R is cut, so this holds for
+// matrices whose unknowns have one scale: they come in equilibrated by powers of two (k_dense.cu), and the last
+// kernel takes the equilibration back.
 #include <cuda_fp16.h>
 
 #include "kernels.h"
@@ -454,13 +457,16 @@ __global__ void k_inv_perm(int N, const int* __restrict__ swp, int* __restrict__
   __syncthreads();
   for (int j = threadIdx.x; j < N; j += blockDim.x) perm[o + j] = pm[j];
 }
-// X[:, perm[j]] = A[:, j]
+// X[i, perm[j]] = 2^ex[i] A[i, j] 2^ex[perm[j]]: the column order, and the equilibration of the matrix taken back
 __global__ void k_inv_columns(int N, const double2* __restrict__ A, const int* __restrict__ perm,
-                              double2* __restrict__ X) {
+                              const int* __restrict__ ex, double2* __restrict__ X) {
   const int mat = blockIdx.z, j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
   if (j >= N) return;
   const long long o = ((long long)mat * N + i) * N;
-  X[o + perm[(long long)mat * N + j]] = A[o + j];
+  const int* es = ex + (long long)mat * N;
+  const int p = perm[(long long)mat * N + j], e = es[i] + es[p];
+  const double2 v = A[o + j];
+  X[o + p] = make_double2(ldexp(v.x, e), ldexp(v.y, e));
 }
 
 struct Plan {
@@ -565,7 +571,7 @@ size_t dense_invert_workspace(int N, int nmat) {
   return 2 * up256(p.dig) + up256(p.gp) + up256(sizeof(int) * (size_t)nmat * 2 * (p.Npad + N));
 }
 
-int dense_invert(int N, int nmat, double2* A, double2* inv, void* ws, int* err, cudaStream_t s) {
+int dense_invert(int N, int nmat, double2* A, const int* ex, double2* inv, void* ws, int* err, cudaStream_t s) {
   const Plan p = plan_for(N, nmat);
   unsigned char* w = (unsigned char*)ws;
   __half* wd = (__half*)w;
@@ -581,7 +587,7 @@ int dense_invert(int N, int nmat, double2* A, double2* inv, void* ws, int* err, 
                     : invert_t<16>(p, N, nmat, A, gp, wd, rd, we, re, swp, err, s);
   cudaFuncSetAttribute(k_inv_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, PERM_SMEM);
   k_inv_perm<<<nmat, 256, 2 * N * sizeof(int), s>>>(N, swp, perm);
-  k_inv_columns<<<dim3((N + 255) / 256, N, nmat), 256, 0, s>>>(N, A, perm, inv);
+  k_inv_columns<<<dim3((N + 255) / 256, N, nmat), 256, 0, s>>>(N, A, perm, ex, inv);
   return n + 2;
 }
 

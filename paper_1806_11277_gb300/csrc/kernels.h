@@ -223,18 +223,24 @@ void launch_prolong_add(const Grid& gf, const Grid& gc, int items, const typenam
                         typename CT<T>::type* xf, cudaStream_t s);
 
 // ---- coarsest level (dense FP64) ----------------------------------------
-void launch_dense_assemble(const Grid& g, int nsets, const StencilLayout& L, const double2* tab,
+// exponents ex [nsets][N] of the equilibration D = diag(2^ex) of the coarsest operator (two launches)
+void launch_dense_scale(const Grid& g, int nsets, const StencilLayout& L, const double2* tab, int* ex,
+                        cudaStream_t s);
+// A = D K_c D
+void launch_dense_assemble(const Grid& g, int nsets, const StencilLayout& L, const double2* tab, const int* ex,
                            double2* A /*[nsets][N][N], zeroed*/, cudaStream_t s);
-// inv = A^{-1} for nmat matrices [N][N] (A is overwritten; ws: dense_invert_workspace bytes); returns the
-// number of launches
+// inv = D A^{-1} D, D = diag(2^ex), for nmat matrices [N][N] with exponents [N] each (A is overwritten; ws:
+// dense_invert_workspace bytes); returns the number of launches
 size_t dense_invert_workspace(int N, int nmat);
-int dense_invert(int N, int nmat, double2* A, double2* inv, void* ws, int* err, cudaStream_t s);
+int dense_invert(int N, int nmat, double2* A, const int* ex, double2* inv, void* ws, int* err, cudaStream_t s);
 template <typename T>
 void launch_dense_apply(int N, int items, int nrhs, const double2* inv, const typename CT<T>::type* r,
                         typename CT<T>::type* x, cudaStream_t s);
-// MG-DD: local dense matrices of the coarsest-grid subdomains ([nsets*nsub][nloc][nloc], zeroed)
+// MG-DD: local dense matrices of the coarsest-grid subdomains ([nsets*nsub][nloc][nloc], zeroed), equilibrated by
+// the coarsest unknowns' exponents ex, and the exponents exl [nsets*nsub][nloc] of their rows
 void launch_dense_assemble_sub(const Grid& g, int nsets, int nsub, int nloc, const StencilLayout& L,
-                               const double2* tab, const int* map, const int* g2l, double2* A, cudaStream_t s);
+                               const double2* tab, const int* ex, const int* map, const int* g2l, double2* A,
+                               int* exl, cudaStream_t s);
 // x = inv r with a low-precision inverse, FP32 accumulation; fmt 1 complex64, 2 FP16 pairs,
 // 3 BF16 pairs; matrix of item b: inv + (b / nrhs) N^2 entries.  sizes (device, optional):
 // live size of matrix set s is sizes[s % nsub], the rest identity padding (skipped)
