@@ -177,7 +177,9 @@ __global__ void __launch_bounds__(PT) k_inv_panel(int N, int Npad, int k0, int b
     const int p = best.y;
     if (rank == 0 && threadIdx.x == 0) {
       swp[(long long)mat * N + k] = p;
-      if (best.x < 0x1e600000) atomicOr(err, EHS_DEVERR_SINGULAR);   // |pivot|^2 below the FP64 range
+      // a pivot whose |.|^2 leaves the FP64 range (below 2^-537, from 2^511 on), or that is not finite: Inf and NaN
+      // rank above every number in the search
+      if (best.x < 0x1e600000 || best.x >= 0x5fe00000) atomicOr(err, EHS_DEVERR_SINGULAR);
     }
     const double2 u = srow[par][win][col];
     bk = -1;

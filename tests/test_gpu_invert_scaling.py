@@ -114,3 +114,14 @@ def test_large_coarsest_solve_inverts_the_coarsest_operator(cells, media):
         # backward stable: |A x - b| <= c N u |A| |A^{-1}| |b|, |A| |A^{-1}| below 1e3 here
         n = 3 * cells[0] * cells[1]
         assert float(((r - b).abs().amax() / b.abs().amax()).cpu()) <= n * 2.0 ** -53 * 1e3
+
+
+# finite media whose operator overflows FP64: setup reports the matrix, with or without subdomains
+@pytest.mark.parametrize("split", [(1, 1, 1), (2, 2, 1)])
+def test_a_coarsest_matrix_that_overflows_is_reported(split):
+    m = synth.random_2d(n=48, nx=56, sigma=0.25, seed=3, corr=4.0, abl=4)
+    f = 1e308 / m.mu.max()
+    huge = synth.Medium(-0.5 * f * m.mu, f * m.mu, m.rho, m.omega, m.h, m.abl_cells)
+    with pytest.raises(ehs.EhsError, match="singular") as e:
+        ehs.solver_for(huge, levels=3, alpha=ALPHA, prec=ehs.EHS_C128, coarse_dd=split, coarse_dd_overlap=2).close()
+    assert ehs.STATUS[e.value.status] == "ERR_ARG"
