@@ -33,18 +33,17 @@ __device__ __forceinline__ void st_one_row(const Grid& g, const TT* ts, long lon
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
-__global__ void __launch_bounds__(256) k_st_rows(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
+__global__ void __launch_bounds__(256) k_st_rows(Grid g, int nrhs, const TT* __restrict__ tab,
                                                  const typename CT<T>::type* x,
                                                  const typename CT<T>::type* b,
                                                  typename CT<T>::type* __restrict__ y, int mode, int colour,
                                                  const int* il) {
   pdl_enter();
   constexpr StencilLayout L = level_layout(D, LV);
-  const unsigned blk = blockIdx.x / (unsigned)nit, it = blockIdx.x - blk * (unsigned)nit;
-  const long long c = (long long)blk * blockDim.x + threadIdx.x;
+  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int a = blockIdx.z;
-  const int item = il ? il[it] : it;
+  const int item = il ? il[blockIdx.y] : blockIdx.y;
   int i[3];
   cell_coords(g, c, i);
   if (a == D && colour >= 0 && ((i[0] + i[1] + i[2]) & 1) != colour) return;
@@ -169,17 +168,16 @@ __device__ __forceinline__ void st_two_rows(const Grid& g, const TT* ts, long lo
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
-__global__ void k_st_rows2(Grid g, int nit, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* x,
+__global__ void k_st_rows2(Grid g, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* x,
                            const typename CT<T>::type* b, typename CT<T>::type* __restrict__ y,
                            int mode, int colour, const int* il) {
   pdl_enter();
   constexpr StencilLayout L = level_layout(D, LV);
-  const unsigned blk = blockIdx.x / (unsigned)nit, it = blockIdx.x - blk * (unsigned)nit;
-  const long long t = (long long)blk * blockDim.x + threadIdx.x;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= g.ncell / 2) return;
   const long long c = 2 * t;
   const int a = blockIdx.z;
-  const int item = il ? il[it] : it;
+  const int item = il ? il[blockIdx.y] : blockIdx.y;
   int i[3];
   cell_coords(g, c, i);
   const long long N = g.ncell;
@@ -203,26 +201,27 @@ static void st_apply_t(const Grid& g, int items, int nrhs, int v, const TT* tab,
                        int var, cudaStream_t s) {
   if (var < 0 || var >= ST_ROWS_VARIANTS || (kRowsCpt[var] == 2 && (g.n[0] & 1))) var = 0;
   const int bs = kRowsBs[var];
-  // the items of a batch take turns on the same cells: their blocks run side by side, and the table
-  // entries they share come from L2 after the first
+  // An item's blocks run together: its vectors, which a row reads at every neighbour, stay in L1 and L2.  With the
+  // items of a batch taking turns on the same cells instead, so that the table entries they share come from L2:
+  // 16 sources of 256^2 on level 1 (complex64 table) 74 -> 118 us, 8 sources of 56 x 44 x 44 (FP16) 323 -> 509.
   const int nit = (int)sel_items(items);
   if (kRowsCpt[var] == 1) {
-    const dim3 gr((unsigned)((g.ncell + bs - 1) / bs) * nit, 1, g.d + 1);
+    const dim3 gr((unsigned)((g.ncell + bs - 1) / bs), nit, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     } else if constexpr (!SYM) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     }
   } else {
-    const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs) * nit, 1, g.d + 1);
+    const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs), nit, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     } else if constexpr (!SYM) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 1, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 2, SYM>, g, nit, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
     }
   }
 }

@@ -1,0 +1,59 @@
+"""Batches large enough for the launch forms of large problems: every item gets what it gets alone."""
+import pytest
+import torch
+
+from paper_1806_11277_gb300 import ehs, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _medium(shape):
+    if len(shape) == 2:
+        return synth.random_2d(n=shape[0], nx=shape[1], sigma=0.3, seed=7, corr=4.0, abl=2)
+    m = synth.layered_3d(n=max(shape), abl=2, corr=3.0)
+    cut = tuple(slice(0, s) for s in shape)
+    return synth.Medium(m.lam[cut], m.mu[cut], m.rho[cut], m.omega, m.h, 2)
+
+
+def _vec(shp, dt, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    v = torch.randn(shp, dtype=torch.complex128, device="cuda", generator=gen)
+    d = len(shp) - 2
+    for k in range(d):
+        v[:, k].select(d - k, 0).zero_()
+    return v.to(dt)
+
+
+def _compare(shape, nrhs, levels, dt, run, tol, **kw):
+    """run(S, n): outputs of the call under test on the first n sources; items 0, 1 and the last against one source."""
+    med = _medium(shape)
+    kw = dict(levels=levels, alpha=0.4, restart=1, **kw)
+    with ehs.solver_for(med, nrhs=nrhs, **kw) as S, ehs.solver_for(med, nrhs=1, **kw) as S1:
+        outs = run(S, lambda l, seed: _vec(S.level_shape(l), dt, seed))
+        for i in (0, 1, nrhs - 1):
+            ones = run(S1, lambda l, seed: _vec(S.level_shape(l), dt, seed)[i:i + 1].contiguous())
+            for a, b in zip(outs, ones):
+                assert float((a[i] - b[0]).abs().max() / b.abs().max()) <= tol, i
+
+
+# residual passes of Galerkin levels, every launch shape: ragged rows, more than one block an item, an odd batch
+@pytest.mark.parametrize("variant", ["0", "1", "2", "3"])
+@pytest.mark.parametrize("shape,nrhs,half", [((72, 104), 5, 0), ((72, 104), 5, 2), ((24, 16, 20), 3, 0),
+                                             ((24, 16, 20), 3, 1)])
+def test_galerkin_rows(shape, nrhs, half, variant, monkeypatch):
+    monkeypatch.setenv("EHS_ROWS_VARIANT", variant)
+
+    def run(S, vec):
+        out = []
+        for l in (1, 2):
+            x, b = vec(l, l), vec(l, 10 + l)
+            y = torch.empty_like(x)
+            S.op_apply(x, y, level=l)
+            out.append(y)
+            if l == 1:
+                S.smooth(b, x, level=l, nsweeps=2)
+                out.append(x)
+        return out
+
+    for dt, tol in ((torch.complex64, 2e-5), (torch.complex128, 1e-12)):   # the bars of an operator and a sweep
+        _compare(shape, nrhs, 3, dt, run, tol, coef_half=half)
