@@ -17,17 +17,27 @@ namespace {
 // a warp and the row's stencil loop is fully unrolled.  mode 0: y = A x,
 // mode 1: y = b - A x.  colour >= 0 restricts the pressure rows to cells of
 // that colour (the rows a red-black half-sweep needs).
+// Rows launched plainly, reading x and b as data that does not change: those of the FP64 form, and of the full complex64
+// tables of 2D levels from 2 on (135 coefficients a cell).  us a residual pass / a sweep, launch_pdl -> plain: FP64
+// 100 x 172, level 1 21.6 / 76 -> 16.7 / 41, three items of 24 x 20 x 28 159 / 361 -> 142 / 309, complex64 four media of
+// 128^2 from level 2 on 22 / 52 -> 15 / 37.  The others lose: complex64 256^2, level 1 8.0 / 22.8 -> 10.5 / 24.6, half tables
+// 18.5 / 44.7 -> 20.7 / 49.2, 3D 48^3 95 / 200 -> 121 / 253.
+template <typename T, int D, int LV, bool SYM> __host__ __device__ constexpr bool plain_rows() {
+  return sizeof(T) == 8 || (D == 2 && LV == 2 && !SYM);
+}
+
 template <typename T, typename TT, int D, int LV, bool SYM, int A>
 __device__ __forceinline__ void st_one_row(const Grid& g, const TT* ts, long long c,
                                            const int i[3], const typename CT<T>::type* xv,
                                            const typename CT<T>::type* bv, typename CT<T>::type* yv,
                                            int mode) {
   typedef typename CT<T>::type Cx;
+  constexpr bool PLAIN = plain_rows<T, D, LV, SYM>();
   const long long N = g.ncell;
   Cx r = czero<Cx>();
   if (slot_valid(A, D, i)) {
-    r = st_row_ct<T, TT, D, LV, SYM, A>(g, ts, c, i, xv);
-    if (mode) r = csub(*(bv + (long long)A * N + c), r);
+    r = st_row_ct<T, TT, D, LV, SYM, A, false, 1, 0, PLAIN>(g, ts, c, i, xv);
+    if (mode) r = csub(ld_vec<PLAIN>(bv + (long long)A * N + c), r);
   }
   yv[(long long)A * N + c] = r;
 }
@@ -96,6 +106,7 @@ __device__ __forceinline__ void row_acc2(typename CT<T>::type& y0, typename CT<T
                                          const typename CT<T>::type* x) {
   if constexpr (Q < QE) {
     typedef typename CT<T>::type Cx;
+    constexpr bool PLAIN = plain_rows<T, D, LV, SYM>();
     constexpr StencilLayout L = level_layout(D, LV);
     constexpr int b = L.p[Q].b, base = L.p[Q].base;
     constexpr int lo0 = L.p[Q].lo[0], lo1 = L.p[Q].lo[1], lo2 = L.p[Q].lo[2];
@@ -135,8 +146,8 @@ __device__ __forceinline__ void row_acc2(typename CT<T>::type& y0, typename CT<T
           } else {
             Pair2<TT>::ld(tab + (long long)(base + ti) * N + c, t0, t1);
           }
-          if (in0) x0 = *(xb + cj);
-          if (in1) x1 = *(xb + cj + 1);
+          if (in0) x0 = ld_vec<PLAIN>(xb + cj);
+          if (in1) x1 = ld_vec<PLAIN>(xb + cj + 1);
           y0 = cfma(t0, x0, y0);
           y1 = cfma(t1, x1, y1);
         }
@@ -151,6 +162,7 @@ __device__ __forceinline__ void st_two_rows(const Grid& g, const TT* ts, long lo
                                             const typename CT<T>::type* xv, const typename CT<T>::type* bv,
                                             typename CT<T>::type* yv, int mode, int colour) {
   typedef typename CT<T>::type Cx;
+  constexpr bool PLAIN = plain_rows<T, D, LV, SYM>();
   constexpr StencilLayout L = level_layout(D, LV);
   const long long N = g.ncell;
   Cx y0 = czero<Cx>(), y1 = czero<Cx>();
@@ -160,8 +172,8 @@ __device__ __forceinline__ void st_two_rows(const Grid& g, const TT* ts, long lo
   const int par = (i[0] + i[1] + i[2]) & 1;
   const bool w0 = !(A == D && colour >= 0 && par != colour), w1 = !(A == D && colour >= 0 && par == colour);
   if (mode) {
-    if (v0) y0 = csub(*(bv + (long long)A * N + c), y0);
-    if (v1) y1 = csub(*(bv + (long long)A * N + c + 1), y1);
+    if (v0) y0 = csub(ld_vec<PLAIN>(bv + (long long)A * N + c), y0);
+    if (v1) y1 = csub(ld_vec<PLAIN>(bv + (long long)A * N + c + 1), y1);
   }
   if (w0) yv[(long long)A * N + c] = v0 ? y0 : czero<Cx>();
   if (w1) yv[(long long)A * N + c + 1] = v1 ? y1 : czero<Cx>();
@@ -195,6 +207,12 @@ __global__ void k_st_rows2(Grid g, int nrhs, const TT* __restrict__ tab, const t
 static const int kRowsCpt[ST_ROWS_VARIANTS] = {1, 2, 1, 2};
 static const int kRowsBs[ST_ROWS_VARIANTS] = {128, 128, 256, 64};
 
+template <bool PLAIN, typename K, typename... A>
+static void launch_rows(dim3 gr, int bs, cudaStream_t s, K kernel, A... args) {
+  if (PLAIN) launch_plain(gr, bs, 0, s, kernel, args..., g_sel.list);
+  else launch_pdl(gr, bs, 0, s, kernel, args..., g_sel.list);
+}
+
 template <typename T, typename TT, bool SYM>
 static void st_apply_t(const Grid& g, int items, int nrhs, int v, const TT* tab, const typename CT<T>::type* x,
                        const typename CT<T>::type* b, typename CT<T>::type* y, int mode, int colour,
@@ -208,20 +226,20 @@ static void st_apply_t(const Grid& g, int items, int nrhs, int v, const TT* tab,
   if (kRowsCpt[var] == 1) {
     const dim3 gr((unsigned)((g.ncell + bs - 1) / bs), nit, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_rows<plain_rows<T, 2, 1, SYM>()>(gr, bs, s, k_st_rows<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 2, 2, SYM>()>(gr, bs, s, k_st_rows<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
     } else if constexpr (!SYM) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_rows<plain_rows<T, 3, 1, SYM>()>(gr, bs, s, k_st_rows<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 3, 2, SYM>()>(gr, bs, s, k_st_rows<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
     }
   } else {
     const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs), nit, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_rows<plain_rows<T, 2, 1, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 2, 2, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
     } else if constexpr (!SYM) {
-      if (v == 1) launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
-      else launch_pdl(gr, bs, 0, s, k_st_rows2<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour, g_sel.list);
+      if (v == 1) launch_rows<plain_rows<T, 3, 1, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 3, 2, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
     }
   }
 }

@@ -51,6 +51,19 @@ inline void launch_pdl(dim3 grid, dim3 block, size_t smem, cudaStream_t s, void 
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// A plain launch of the same kernels: it starts when its inputs are complete, so that what earlier launches wrote may be read as
+// data that does not change (__ldg).  Compilers move such loads freely and the long loops of FP64 rows and products
+// need it; a launch_pdl kernel pays for that with plain loads what it saves in launch time.
+template <typename... P, typename... A>
+inline void launch_plain(dim3 grid, dim3 block, size_t smem, cudaStream_t s, void (*kernel)(P...), A... args) {
+  kernel<<<grid, block, smem, s>>>(static_cast<P>(args)...);
+}
+// vector entries of a kernel launched plainly (PLAIN) or by launch_pdl
+template <bool PLAIN, typename C> __device__ __forceinline__ C ld_vec(const C* p) {
+  if constexpr (PLAIN) return __ldg(p);
+  else return *p;
+}
+
 // Threads per block of a one-thread-per-unit launch of n units per item: bs, halved down to one warp while
 // the blocks do not reach every SM.  A small launch is bound by what one SM does (above all by its FP64 pipe: 2
 // lanes a clock), not by the number of blocks: one FP64 colour of 64^2 cells 15.5 us on 16 SMs.

@@ -52,10 +52,12 @@ __device__ __forceinline__ int half_slot_of(int ti, bool& mir) {
 // known at compile time so that every table and vector load of the row is
 // issued back to back.  SYM: the table is stored half (common.cuh HalfMap), an
 // unstored coefficient read from its mirror at the neighbour cell.
-// XCG: x is read through L2 only (x written earlier by the same launch on other SMs).
+// XCG: x is read through L2 only (x written earlier by the same launch on other SMs).  PLAIN: the kernel is launched
+// plainly and reads x as data that does not change.
 // NS > 1: only the coefficients whose slot index is SI modulo NS (a share of the row, the
 // rest summed by NS - 1 other threads).
-template <typename T, typename TT, int D, int LV, bool SYM, int Q, int QE, bool XCG = false, int NS = 1, int SI = 0>
+template <typename T, typename TT, int D, int LV, bool SYM, int Q, int QE, bool XCG = false, int NS = 1, int SI = 0,
+          bool PLAIN = false>
 __device__ __forceinline__ void row_acc(typename CT<T>::type& y, const Grid& g,
                                         const TT* __restrict__ tab,
                                         long long c, const int i[3],
@@ -95,23 +97,24 @@ __device__ __forceinline__ void row_acc(typename CT<T>::type& y, const Grid& g,
             } else {
               tv = ldtab<T>(tab + (long long)(base + ti) * N + c);
             }
-            if (in) xv = XCG ? __ldcg(xb + cj) : *(xb + cj);
+            if (in) xv = XCG ? __ldcg(xb + cj) : ld_vec<PLAIN>(xb + cj);
             y = cfma(tv, xv, y);
           }
         }
       }
     }
-    row_acc<T, TT, D, LV, SYM, Q + 1, QE, XCG, NS, SI>(y, g, tab, c, i, x);
+    row_acc<T, TT, D, LV, SYM, Q + 1, QE, XCG, NS, SI, PLAIN>(y, g, tab, c, i, x);
   }
 }
 
-template <typename T, typename TT, int D, int LV, bool SYM, int A, bool XCG = false, int NS = 1, int SI = 0>
+template <typename T, typename TT, int D, int LV, bool SYM, int A, bool XCG = false, int NS = 1, int SI = 0,
+          bool PLAIN = false>
 __device__ __forceinline__ typename CT<T>::type st_row_ct(const Grid& g, const TT* tab,
                                                            long long c, const int i[3],
                                                            const typename CT<T>::type* x) {
   constexpr StencilLayout L = level_layout(D, LV);
   typename CT<T>::type y = czero<typename CT<T>::type>();
-  row_acc<T, TT, D, LV, SYM, L.row_first[A], L.row_first[A + 1], XCG, NS, SI>(y, g, tab, c, i, x);
+  row_acc<T, TT, D, LV, SYM, L.row_first[A], L.row_first[A + 1], XCG, NS, SI, PLAIN>(y, g, tab, c, i, x);
   return y;
 }
 
