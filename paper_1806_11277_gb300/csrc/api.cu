@@ -568,7 +568,7 @@ void autotune_rows(ehs_ctx* c, Hier& H) {
     Level& L = H.lv[l];
     int fmt = 0;
     const void* tab = tabp<T>(H, L, &fmt);
-    if (st_split(L.g, H.items, layout_variant(L.L, L.g.d), fmt)) {   // by size alone
+    if (st_split(L.g, H.items, H.nrhs, layout_variant(L.L, L.g.d), fmt, p == 0)) {   // by size alone
       L.rows_var[p] = ST_ROWS_SPLIT;
       continue;
     }

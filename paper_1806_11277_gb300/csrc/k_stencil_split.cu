@@ -156,7 +156,8 @@ __global__ void __launch_bounds__(32 * NS) k_st_rows_split(Grid g, int nit, int 
 
 // The 3D form: NI items of the list per block, one read of the table for all of them where they are of one medium
 // (its coefficients are nine tenths of the bytes; 64^3, complex64 tables, two sources, mean of levels 1 and 2: 43 us with an
-// item a block, the table read once per item -> 30 us).
+// item a block, the table read once per item -> 30 us).  The FP64 form keeps an item a block: its pipe bounds it, not the
+// table (16^3 from level 2 on, three items: 102 us, 143 with two items a block).
 template <typename T, typename TT, int LV, int NS, int NI>
 __global__ void __launch_bounds__(32 * NS) k_st_rows_split3(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
                                                             const typename CT<T>::type* x,
@@ -387,12 +388,15 @@ void rows_split_t(const Grid& g, int items, int nrhs, const TT* tab, const typen
   const int nit = (int)sel_items(items);
   const unsigned nb = (unsigned)((g.ncell + 31) / 32);
   if constexpr (D == 3) {
-    if (nrhs > 1)
-      launch_pdl(dim3(nb * ((nit + 1) / 2), 1, 4), 32 * NS, 0, s, k_st_rows_split3<T, TT, LV, NS, 2>, g, nit, nrhs, tab, x,
-                 b, y, mode, colour, g_sel.list);
-    else
-      launch_pdl(dim3(nb * nit, 1, 4), 32 * NS, 0, s, k_st_rows_split3<T, TT, LV, NS, 1>, g, nit, nrhs, tab, x, b, y, mode,
-                 colour, g_sel.list);
+    if constexpr (sizeof(T) == 4) {
+      if (nrhs > 1) {
+        launch_pdl(dim3(nb * ((nit + 1) / 2), 1, 4), 32 * NS, 0, s, k_st_rows_split3<T, TT, LV, NS, 2>, g, nit, nrhs,
+                   tab, x, b, y, mode, colour, g_sel.list);
+        return;
+      }
+    }
+    launch_pdl(dim3(nb * nit, 1, 4), 32 * NS, 0, s, k_st_rows_split3<T, TT, LV, NS, 1>, g, nit, nrhs, tab, x, b, y, mode,
+               colour, g_sel.list);
   } else {
     launch_pdl(dim3(nb * nit, 1, 3), 32 * NS, 0, s, k_st_rows_split<T, TT, D, LV, SYM, NS>, g, nit, nrhs, tab, x, b, y,
                mode, colour, g_sel.list);
@@ -442,15 +446,16 @@ void colour_d(int v, const TT* tab, const Grid& g, int items, int nrhs, const fl
 //   32^2: 6.4 -> 4.2; above, 256^2: 8.5 -> 12.5
 //   3D, from level 2 on: every size measured (16^3 40 -> 12, two items of 24^3 158 -> 43, FP16 tables 62 -> 39);
 //   3D, level 1 (rows half as long): 16^3 21 -> 8, 32^3 with complex64 tables 52 -> 35 and two items 66 -> 62, but
-//   with FP16 tables 21 -> 31; 48^3 97 -> 105
+//   with FP16 tables 21 -> 31; 48^3 97 -> 105; an odd batch fills only half of its last pair of items (three of
+//   24 x 20 x 28: 25 -> 29).  FP64: 16^3 39 -> 27, but two items 41 -> 44, 24 x 20 x 28 64 -> 64, 32^3 128 -> 149.
 // and a sweep of the 2D complex64 cycle with one launch per colour instead of two: 128^2 24.8 -> 16.9 us (complex64
 // table), 28.9 -> 20.4 (FP16, level 2 on), 64^2 24.8 -> 12.4; not at 256^2 (31 -> 33 to 50) nor for 16 items of 64^2
 // (40 -> 49).  The FP64 cycle keeps two launches (53 -> 62 at 128^2: one warp of the block would do all of the
 // block solve's FP64 arithmetic).
-bool st_split(const Grid& g, int items, int v, int fmt) {
+bool st_split(const Grid& g, int items, int nrhs, int v, int fmt, bool fp64) {
   const long long cells = (long long)items * g.ncell;
   if (g.d == 2) return cells <= 16384;
-  return v != 1 || cells <= (fmt ? 16384 : 65536);
+  return v != 1 || cells <= (fp64 ? 4096 : fmt ? 16384 : nrhs > 1 && nrhs % 2 ? 32768 : 65536);
 }
 template <typename T>
 void launch_st_rows_split(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt,

@@ -173,7 +173,7 @@ int layout_variant(const StencilLayout& L, int d);
 // colour >= 0: pressure rows of that colour only)
 // ST_ROWS_SPLIT: rows split over the warps of a block, and one colour's relaxation in one launch (2D complex64
 // cycle); k_stencil_split.cu
-bool st_split(const Grid& g, int items, int v, int fmt);
+bool st_split(const Grid& g, int items, int nrhs, int v, int fmt, bool fp64);
 template <typename T>
 void launch_st_rows_split(const Grid& g, int items, int nrhs, int v, const void* tab, int fmt,
                           const typename CT<T>::type* x, const typename CT<T>::type* b, typename CT<T>::type* y,

@@ -57,3 +57,29 @@ def test_galerkin_rows(shape, nrhs, half, variant, monkeypatch):
 
     for dt, tol in ((torch.complex64, 2e-5), (torch.complex128, 1e-12)):   # the bars of an operator and a sweep
         _compare(shape, nrhs, 3, dt, run, tol, coef_half=half)
+
+
+# 3D rows split over warps, two items a block: a last block with one item, pairs that straddle two media, sizes on both
+# sides of the limits of the split form (FP64 4096 cells of the batch, FP16 tables 16384, an odd batch 32768)
+@pytest.mark.parametrize("half", [0, 1])
+@pytest.mark.parametrize("shape,media,nrhs", [((16, 16, 8), 1, 3), ((16, 16, 8), 2, 3), ((32, 16, 32), 1, 3),
+                                              ((48, 40, 48), 1, 3)])
+def test_split_rows_of_odd_batches(shape, media, nrhs, half, monkeypatch):
+    m = _medium(shape)
+    meds = [synth.Medium(m.lam * (1 + 0.2 * k), m.mu, m.rho * (1 - 0.1 * k), m.omega, m.h, 2) for k in range(media)]
+    got = []
+    for fixed in (None, "0"):
+        if fixed is not None:
+            monkeypatch.setenv("EHS_ROWS_VARIANT", fixed)
+        out = []
+        with ehs.solver_for(meds, levels=3, alpha=0.4, nrhs=nrhs, coef_half=half, restart=1) as S:
+            for dt in (torch.complex64, torch.complex128):
+                for l in (1, 2):
+                    x = _vec(S.level_shape(l), dt, l)
+                    y = torch.empty_like(x)
+                    S.op_apply(x, y, level=l)
+                    out.append(y)
+        got.append(out)
+    for a, b in zip(*got):                    # the same sums in another order: the bars of the operator
+        tol = 1e-5 if a.dtype == torch.complex64 else 1e-12
+        assert float((a - b).abs().max() / b.abs().max()) <= tol
