@@ -83,3 +83,14 @@ def test_split_rows_of_odd_batches(shape, media, nrhs, half, monkeypatch):
     for a, b in zip(*got):                    # the same sums in another order: the bars of the operator
         tol = 1e-5 if a.dtype == torch.complex64 else 1e-12
         assert float((a - b).abs().max() / b.abs().max()) <= tol
+
+
+# complex64 prolongations above 400 K cells of the batch run a thread per cell instead of per component
+@pytest.mark.parametrize("shape,nrhs", [((136, 120), 25), ((24, 16, 20), 55)])
+def test_prolongation(shape, nrhs):
+    def run(S, vec):
+        x = vec(0, 1)
+        S.prolong_add(vec(1, 2), x)
+        return [x]
+
+    _compare(shape, nrhs, 3, torch.complex64, run, 1e-5)
