@@ -112,8 +112,10 @@ __global__ void k_dense_assemble(Grid g, StencilLayout L, const double2* __restr
   }
 }
 
-// x = Ainv r, one warp per dense row; input/output in the working precision
-template <typename T>
+// x = Ainv r, one warp per dense row; input/output in the working precision.  Bound by the FP64 pipe.  PLAIN: launched
+// plainly, r read as data that does not change, so that the loop's loads run ahead (N = 3072 82 us, 123 with
+// launch_pdl, 100 with four of its loads issued together by hand)
+template <typename T, bool PLAIN>
 __global__ void k_dense_apply(int N, int nrhs, const double2* __restrict__ inv,
                               const typename CT<T>::type* r,
                               typename CT<T>::type* __restrict__ x, const int* il) {
@@ -127,7 +129,7 @@ __global__ void k_dense_apply(int N, int nrhs, const double2* __restrict__ inv,
   double sx = 0.0, sy = 0.0;
   for (int j = lane; j < N; j += 32) {
     const double2 a = __ldg(row + j);
-    const typename CT<T>::type b = *(rv + j);
+    const typename CT<T>::type b = ld_vec<PLAIN>(rv + j);
     sx = fma(a.x, (double)b.x, fma(-a.y, (double)b.y, sx));
     sy = fma(a.x, (double)b.y, fma(a.y, (double)b.x, sy));
   }
@@ -322,7 +324,12 @@ void launch_dense_apply(int N, int items, int nrhs, const double2* inv, const ty
                         typename CT<T>::type* x, cudaStream_t s) {
   const int wpb = 8;
   dim3 grid((N + wpb - 1) / wpb, sel_items(items));
-  launch_pdl(grid, 32 * wpb, 0, s, k_dense_apply<T>, N, nrhs, inv, r, x, g_sel.list);
+  // from 2048 rows of the batch on the loop counts, below it the launch (N = 768: 9.8 us by launch_pdl, 10.7 plain; four
+  // items of it 33.4 and 24.6)
+  if ((long long)N * sel_items(items) >= 2048)
+    launch_plain(grid, 32 * wpb, 0, s, k_dense_apply<T, true>, N, nrhs, inv, r, x, g_sel.list);
+  else
+    launch_pdl(grid, 32 * wpb, 0, s, k_dense_apply<T, false>, N, nrhs, inv, r, x, g_sel.list);
 }
 
 void launch_dense_assemble_sub(const Grid& g, int nsets, int nsub, int nloc, const StencilLayout& L,

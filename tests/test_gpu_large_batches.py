@@ -94,3 +94,15 @@ def test_prolongation(shape, nrhs):
         return [x]
 
     _compare(shape, nrhs, 3, torch.complex64, run, 1e-5)
+
+
+# FP64 products with the coarsest inverses: plain launches from 2048 rows of the batch on (11 items of 192 rows)
+@pytest.mark.parametrize("split", [(1, 1, 1), (2, 2, 1)])
+def test_fp64_coarsest_products(split):
+    def run(S, vec):
+        b = vec(2, 3)
+        x = torch.empty_like(b)
+        S.coarse_solve(b, x)
+        return [x]
+
+    _compare((32, 32), 11, 3, torch.complex128, run, 1e-10, prec=ehs.EHS_C128, coarse_dd=split, coarse_dd_overlap=1)
