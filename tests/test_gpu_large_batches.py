@@ -106,3 +106,16 @@ def test_fp64_coarsest_products(split):
         return [x]
 
     _compare((32, 32), 11, 3, torch.complex128, run, 1e-10, prec=ehs.EHS_C128, coarse_dd=split, coarse_dd_overlap=1)
+
+
+# the complex64 operator: a plain launch above 1.5 M cells of the batch in 3D
+@pytest.mark.parametrize("shape,nrhs", [((24, 16, 20), 197)])
+def test_complex64_operator(shape, nrhs):
+    def run(S, vec):
+        x, b = vec(0, 1), vec(0, 2)
+        y, r = torch.empty_like(x), torch.empty(S.level_shape(1), dtype=x.dtype, device=x.device)
+        S.op_apply(x, y)
+        S.residual_restrict(b, x, r)
+        return [y, r]
+
+    _compare(shape, nrhs, 3, torch.complex64, run, 1e-5)
