@@ -17,13 +17,32 @@ namespace {
 // a warp and the row's stencil loop is fully unrolled.  mode 0: y = A x,
 // mode 1: y = b - A x.  colour >= 0 restricts the pressure rows to cells of
 // that colour (the rows a red-black half-sweep needs).
+
 // Rows launched plainly, reading x and b as data that does not change: those of the FP64 form, and of the full complex64
 // tables of 2D levels from 2 on (135 coefficients a cell).  us a residual pass / a sweep, launch_pdl -> plain: FP64
 // 100 x 172, level 1 21.6 / 76 -> 16.7 / 41, three items of 24 x 20 x 28 159 / 361 -> 142 / 309, complex64 four media of
-// 128^2 from level 2 on 22 / 52 -> 15 / 37.  The others lose: complex64 256^2, level 1 8.0 / 22.8 -> 10.5 / 24.6, half tables
+// 128^2 from level 2 on 22 / 52 -> 14.6 / 33.  The others lose: complex64 256^2, level 1 8.0 / 22.8 -> 10.5 / 24.6, half tables
 // 18.5 / 44.7 -> 20.7 / 49.2, 3D 48^3 95 / 200 -> 121 / 253.
 template <typename T, int D, int LV, bool SYM> __host__ __device__ constexpr bool plain_rows() {
   return sizeof(T) == 8 || (D == 2 && LV == 2 && !SYM);
+}
+
+// An item's blocks follow one another: its vectors, which a row reads at every neighbour, stay in L1 and L2.  With the
+// items of a batch taking turns on the same cells instead, so that the table entries they share come from L2:
+// 16 sources of 256^2 on level 1 (complex64 table) 74 -> 118 us, 8 sources of 56 x 44 x 44 (FP16) 323 -> 509.  The
+// item is blockIdx.y, in 2D with a full table counted out of blockIdx.x: the row's code comes out differently (complex64 100 x 172
+// a sweep 17.2 -> 16.3 us counted out, 48^3 200 -> 252).
+struct Blk {
+  unsigned blk, it;
+};
+template <int D, bool SYM> __host__ __device__ constexpr bool flat_rows() { return D == 2 && !SYM; }
+template <int D, bool SYM> __device__ __forceinline__ Blk block_of(unsigned nblk) {
+  if constexpr (flat_rows<D, SYM>()) {
+    const unsigned it = blockIdx.x / nblk;
+    return {blockIdx.x - it * nblk, it};
+  } else {
+    return {blockIdx.x, blockIdx.y};
+  }
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM, int A>
@@ -43,17 +62,18 @@ __device__ __forceinline__ void st_one_row(const Grid& g, const TT* ts, long lon
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
-__global__ void __launch_bounds__(256) k_st_rows(Grid g, int nrhs, const TT* __restrict__ tab,
+__global__ void __launch_bounds__(256) k_st_rows(Grid g, unsigned nblk, int nrhs, const TT* __restrict__ tab,
                                                  const typename CT<T>::type* x,
                                                  const typename CT<T>::type* b,
                                                  typename CT<T>::type* __restrict__ y, int mode, int colour,
                                                  const int* il) {
   pdl_enter();
   constexpr StencilLayout L = level_layout(D, LV);
-  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const Blk B = block_of<D, SYM>(nblk);
+  const long long c = (long long)B.blk * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int a = blockIdx.z;
-  const int item = il ? il[blockIdx.y] : blockIdx.y;
+  const int item = il ? il[B.it] : B.it;
   int i[3];
   cell_coords(g, c, i);
   if (a == D && colour >= 0 && ((i[0] + i[1] + i[2]) & 1) != colour) return;
@@ -146,10 +166,15 @@ __device__ __forceinline__ void row_acc2(typename CT<T>::type& y0, typename CT<T
           } else {
             Pair2<TT>::ld(tab + (long long)(base + ti) * N + c, t0, t1);
           }
-          if (in0) x0 = ld_vec<PLAIN>(xb + cj);
-          if (in1) x1 = ld_vec<PLAIN>(xb + cj + 1);
-          y0 = cfma(t0, x0, y0);
-          y1 = cfma(t1, x1, y1);
+          if constexpr (PLAIN && sizeof(T) == 4) {   // as in row_acc
+            if (in0) y0 = cfma(t0, ld_vec<PLAIN>(xb + cj), y0);
+            if (in1) y1 = cfma(t1, ld_vec<PLAIN>(xb + cj + 1), y1);
+          } else {
+            if (in0) x0 = ld_vec<PLAIN>(xb + cj);
+            if (in1) x1 = ld_vec<PLAIN>(xb + cj + 1);
+            y0 = cfma(t0, x0, y0);
+            y1 = cfma(t1, x1, y1);
+          }
         }
       }
     }
@@ -180,16 +205,17 @@ __device__ __forceinline__ void st_two_rows(const Grid& g, const TT* ts, long lo
 }
 
 template <typename T, typename TT, int D, int LV, bool SYM>
-__global__ void k_st_rows2(Grid g, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* x,
+__global__ void k_st_rows2(Grid g, unsigned nblk, int nrhs, const TT* __restrict__ tab, const typename CT<T>::type* x,
                            const typename CT<T>::type* b, typename CT<T>::type* __restrict__ y,
                            int mode, int colour, const int* il) {
   pdl_enter();
   constexpr StencilLayout L = level_layout(D, LV);
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const Blk B = block_of<D, SYM>(nblk);
+  const long long t = (long long)B.blk * blockDim.x + threadIdx.x;
   if (t >= g.ncell / 2) return;
   const long long c = 2 * t;
   const int a = blockIdx.z;
-  const int item = il ? il[blockIdx.y] : blockIdx.y;
+  const int item = il ? il[B.it] : B.it;
   int i[3];
   cell_coords(g, c, i);
   const long long N = g.ncell;
@@ -219,27 +245,25 @@ static void st_apply_t(const Grid& g, int items, int nrhs, int v, const TT* tab,
                        int var, cudaStream_t s) {
   if (var < 0 || var >= ST_ROWS_VARIANTS || (kRowsCpt[var] == 2 && (g.n[0] & 1))) var = 0;
   const int bs = kRowsBs[var];
-  // An item's blocks run together: its vectors, which a row reads at every neighbour, stay in L1 and L2.  With the
-  // items of a batch taking turns on the same cells instead, so that the table entries they share come from L2:
-  // 16 sources of 256^2 on level 1 (complex64 table) 74 -> 118 us, 8 sources of 56 x 44 x 44 (FP16) 323 -> 509.
-  const int nit = (int)sel_items(items);
+  const unsigned nit = sel_items(items);
+  const long long nthr = kRowsCpt[var] == 1 ? g.ncell : g.ncell / 2;
+  const unsigned nblk = (unsigned)((nthr + bs - 1) / bs);
+  const dim3 gr = g.d == 2 && !SYM ? dim3(nblk * nit, 1, g.d + 1) : dim3(nblk, nit, g.d + 1);
   if (kRowsCpt[var] == 1) {
-    const dim3 gr((unsigned)((g.ncell + bs - 1) / bs), nit, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) launch_rows<plain_rows<T, 2, 1, SYM>()>(gr, bs, s, k_st_rows<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
-      else launch_rows<plain_rows<T, 2, 2, SYM>()>(gr, bs, s, k_st_rows<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      if (v == 1) launch_rows<plain_rows<T, 2, 1, SYM>()>(gr, bs, s, k_st_rows<T, TT, 2, 1, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 2, 2, SYM>()>(gr, bs, s, k_st_rows<T, TT, 2, 2, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
     } else if constexpr (!SYM) {
-      if (v == 1) launch_rows<plain_rows<T, 3, 1, SYM>()>(gr, bs, s, k_st_rows<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
-      else launch_rows<plain_rows<T, 3, 2, SYM>()>(gr, bs, s, k_st_rows<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      if (v == 1) launch_rows<plain_rows<T, 3, 1, SYM>()>(gr, bs, s, k_st_rows<T, TT, 3, 1, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 3, 2, SYM>()>(gr, bs, s, k_st_rows<T, TT, 3, 2, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
     }
   } else {
-    const dim3 gr((unsigned)((g.ncell / 2 + bs - 1) / bs), nit, g.d + 1);
     if (g.d == 2) {
-      if (v == 1) launch_rows<plain_rows<T, 2, 1, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 2, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
-      else launch_rows<plain_rows<T, 2, 2, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 2, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      if (v == 1) launch_rows<plain_rows<T, 2, 1, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 2, 1, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 2, 2, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 2, 2, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
     } else if constexpr (!SYM) {
-      if (v == 1) launch_rows<plain_rows<T, 3, 1, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 3, 1, SYM>, g, nrhs, tab, x, b, y, mode, colour);
-      else launch_rows<plain_rows<T, 3, 2, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 3, 2, SYM>, g, nrhs, tab, x, b, y, mode, colour);
+      if (v == 1) launch_rows<plain_rows<T, 3, 1, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 3, 1, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
+      else launch_rows<plain_rows<T, 3, 2, SYM>()>(gr, bs, s, k_st_rows2<T, TT, 3, 2, SYM>, g, nblk, nrhs, tab, x, b, y, mode, colour);
     }
   }
 }
