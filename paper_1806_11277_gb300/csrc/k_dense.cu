@@ -8,8 +8,8 @@
 // inverse is scaled back by D from both sides (k_invert.cu): exact scalings, and what is inverted no longer depends
 // on the units of the medium.  Displacements and pressures differ in scale by sqrt(mu (lambda + mu)) / h, near 1
 // in km, km/s and g/cm^3 with h = 1 and about 2^30 in SI units with h = 10 m, and the inverse's digits hold the entries of a
-// row to 2^-55 of the largest: without D the inverse of an SI medium (12 x 14 coarsest cells) is off by 2.5e-8, with
-// it by 1.2e-15 (numpy restatement; FP64 elimination column by column 2.5e-15 in either units).
+// row to 2^-55 of the largest: without D the inverse of an SI medium (12 x 14 coarsest cells) is off by 2.7e-8, with
+// it by 1.3e-15 (numpy restatement; FP64 elimination column by column 2.9e-15).
 //
 // MG-DD (Sec. 4): the same machinery for the subdomains of the coarsest grid.
 // Each box's local matrix (the coarsest operator restricted to the box

@@ -19,8 +19,10 @@
 // matrix multiplication by using fast routines of matrix multiplication and its
 // applications", Numerical Algorithms 2012): every row of W and column of R is scaled
 // by a power of two and cut into six balanced 9-bit digits (55 bits with the sign),
-// digit products of one weight 2^{-9 (i + j)} are summed exactly in the FP32
-// accumulators (|digit| <= 2^8, 2 B products per pair), and the sums of i + j <= 6
+// digit products of one weight 2^{-9 (i + j)} are summed in the FP32 accumulators (|digit| <= 2^8, 2 B products per
+// pair of digits: exactly up to i + j = 3 at B = 32, four pairs of 2^22, and at B = 16 throughout; the five or six pairs of the
+// lower weights could pass 2^24 with nearly every digit at its largest, and would then lose the last unit of
+// 2^{-54} and below), and the sums of i + j <= 6
 // are joined in 64-bit integers before one rounding to FP64.  On the line's box
 // matrices the inverse's error against an 80-bit one is about half that of the
 // FP64 column-by-column elimination (numpy restatement, N = 645: 4.0e-15 against
@@ -505,12 +507,12 @@ template <int B> int clusters_of(int cl, size_t sm) {   // clusters of cl CTAs t
 }
 // B = 32 columns a block up to N = 3200, else 16 (the panel's FP64 work halves, the update's passes over A double).
 // The panel is bound by the FP64 pipe of its SMs, so the cluster size is the one with the fewest rows per CTA
-// times waves of clusters, at one CTA per SM (at least 100 KB of shared memory each: two to an SM, as clusters of
-// 8 with 90 KB were placed, share its pipe).  GB300 runs 7 clusters of 16, 15 of 8, 23 of 6 or 36 of 4 that way.
+// times waves of clusters, at one CTA per SM (at least 110 KB of shared memory each beside 9 to 17 KB of fixed arrays:
+// two to an SM, as clusters of 8 with 90 KB were placed, share its pipe).  GB300 runs 7 clusters of 16, 15 of 8, 23 of 6 or 36 of 4 that way.
 // 16 matrices of 1408: 455 us a block with clusters of 8, two to an SM; 511 with 15 of the 16 at a time; 339 with 6.
 Plan plan_for(int N, int nmat) {
   Plan p;
-  const size_t lim = PANEL_SMEM, least = 100 * 1024;
+  const size_t lim = PANEL_SMEM, least = 110 * 1024;
   p.B = N <= 3200 ? 32 : 16;
   p.Npad = (N + TM - 1) / TM * TM;
   p.cl = 0;
