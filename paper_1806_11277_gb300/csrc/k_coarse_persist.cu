@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(CP_T, EHS_CP_MINBLOCKS) k_coarse_dd_persist(Co
         const long long bl = set * A.nrhs + r;
         const int n = A.sizes[s];
         if (row0 >= n) continue;                       // warp-uniform
-        // r_loc through L1 (__ldg): the sub-items of a colour are first read here, after this
+        // r_loc through L1 (plain loads): the sub-items of a colour are first read here, after this
         // launch wrote them, so no SM holds an older copy (a local vector is a whole number of
         // 32-byte sectors: nloc is a multiple of 8)
         dense_rows4<TI, false, true>(nloc, n, row0, (const TI*)A.inv + set * nloc * nloc, A.rs + bl * nloc,

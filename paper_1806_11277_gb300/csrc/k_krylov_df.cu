@@ -7,7 +7,8 @@
 //
 // Launched plainly (a kernel starts when its inputs are complete), so that the passes over the basis may read it as
 // data that does not change (dfc_ld): with the plain loads of launch_pdl kernels the update pass took 52.9 us instead
-// of 37.5 (two media of 512^2).  The kernels of an Arnoldi step let their successors become resident early.
+// of 37.5 (two media of 512^2).  The last pass of a step (k_dupdate_df) lets the first kernel of the next cycle become
+// resident early.
 //
 // Layouts: Krylov basis V and solution x as complex df64 (float4 per value),
 // preconditioned directions Z as complex64 (the multigrid cycle's output
@@ -352,7 +353,6 @@ template <int NS>
 __global__ void __launch_bounds__(KB, 2) k_mdot2_df(long long n, int items, const float4* __restrict__ V,
                                                  const float4* __restrict__ w, float4* part, int nblk,
                                                  const int* __restrict__ il, int* cnt, float4* coef, double2* outd) {
-  pdl_trigger();
   constexpr int NO = NS + 1;   // NS dots and one norm per half
   static_assert(NO <= MAXV, "sums per half");
   const int item = il ? il[blockIdx.y] : blockIdx.y;
@@ -711,7 +711,6 @@ __global__ void k_fine_apply_df2t(Grid g, int nrhs, const Coef4df* __restrict__ 
                                   const float2* __restrict__ vmt, FinePdf P, const V* __restrict__ x,
                                   const float4* __restrict__ b, float4* __restrict__ y, int mode,
                                   const int* __restrict__ il) {
-  pdl_trigger();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int item = il ? il[blockIdx.y] : blockIdx.y;
@@ -759,7 +758,6 @@ template <typename V, int D>
 __global__ void k_fine_apply_df(Grid g, int nrhs, const Coef4df* __restrict__ cf, FinePdf P,
                                 const V* __restrict__ x, const float4* __restrict__ b,
                                 float4* __restrict__ y, int mode, const int* __restrict__ il) {
-  pdl_trigger();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int item = il ? il[blockIdx.y] : blockIdx.y;

@@ -111,10 +111,9 @@ __device__ __forceinline__ typename CT<T>::type row_part(const Grid& g, const TT
     return czero<typename CT<T>::type>();
   }
 }
-template <typename T, typename TT, int D, int LV, bool SYM, int NS>
+template <typename T, typename TT, int LV, bool SYM, int NS>
 __device__ __forceinline__ typename CT<T>::type row_share(const Grid& g, const TT* ts, long long c, const int i[3],
                                                           const typename CT<T>::type* x, int a, int part) {
-  static_assert(D == 2, "3D rows go by lines");
   if (a == 0) return row_part<T, TT, LV, SYM, NS, 0>(g, ts, c, i, x, part);
   if (a == 1) return row_part<T, TT, LV, SYM, NS, 1>(g, ts, c, i, x, part);
   return row_part<T, TT, LV, SYM, NS, 2>(g, ts, c, i, x, part);
@@ -144,7 +143,7 @@ __global__ void __launch_bounds__(32 * NS) k_st_rows_split(Grid g, int nit, int 
     run = !(a == D && colour >= 0 && ((i[0] + i[1] + i[2]) & 1) != colour);
   }
   const bool row = run && slot_valid(a, D, i);
-  sp[part][lane] = row ? row_share<T, TT, D, LV, SYM, NS>(g, ts, c, i, x + vo, a, part) : czero<Cx>();
+  sp[part][lane] = row ? row_share<T, TT, LV, SYM, NS>(g, ts, c, i, x + vo, a, part) : czero<Cx>();
   __syncthreads();
   if (part || !run) return;
   Cx r = sp[0][lane];
@@ -157,7 +156,7 @@ __global__ void __launch_bounds__(32 * NS) k_st_rows_split(Grid g, int nit, int 
 // The 3D form: NI items of the list per block, one read of the table for all of them where they are of one medium
 // (its coefficients are nine tenths of the bytes; 64^3, complex64 tables, two sources, mean of levels 1 and 2: 43 us with an
 // item a block, the table read once per item -> 30 us).  The FP64 form keeps an item a block: its pipe bounds it, not the
-// table (16^3 from level 2 on, three items: 102 us, 143 with two items a block).
+// table (16^3 from level 2 on, three items: 94 us, 143 with two items a block).
 template <typename T, typename TT, int LV, int NS, int NI>
 __global__ void __launch_bounds__(32 * NS) k_st_rows_split3(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
                                                             const typename CT<T>::type* x,
@@ -222,17 +221,17 @@ __global__ void __launch_bounds__(32 * NS) k_st_rows_split3(Grid g, int nit, int
   y[o] = r;
 }
 
-template <typename T, typename TT, int D, int LV, bool SYM, int NS>
-__global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int nit, int nrhs,
-                                                                     const TT* __restrict__ tab,
-                                                                     const typename CT<T>::type* __restrict__ vtab,
-                                                                     T wu, T wp, int colour,
-                                                                     const typename CT<T>::type* b,
-                                                                     const typename CT<T>::type* xi,
-                                                                     typename CT<T>::type* __restrict__ xo,
-                                                                     const int* il) {
+template <typename T, typename TT, int LV, bool SYM, int NS>
+__global__ void __launch_bounds__(32 * 5 * NS) k_st_colour(Grid g, int nit, int nrhs, const TT* __restrict__ tab,
+                                                           const typename CT<T>::type* __restrict__ vtab,
+                                                           T wu, T wp, int colour,
+                                                           const typename CT<T>::type* b,
+                                                           const typename CT<T>::type* xi,
+                                                           typename CT<T>::type* __restrict__ xo,
+                                                           const int* il) {
   pdl_trigger();
   typedef typename CT<T>::type Cx;
+  constexpr int D = 2;
   constexpr StencilLayout L = level_layout(D, LV);
   constexpr int NB = 2 * D + 1;
   __shared__ Cx sp[NB][NS][32];
@@ -265,8 +264,6 @@ __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int
     }
     vupd_coefs<T, TT, D, LV, SYM, 0>(ts, vt, N, c, stride_of(g, 0), ok[0], ok[D], dinv, gr, gc);
     vupd_coefs<T, TT, D, LV, SYM, 1>(ts, vt, N, c, stride_of(g, 1), ok[1], ok[D + 1], dinv, gr, gc);
-    if constexpr (D == 3)
-      vupd_coefs<T, TT, D, LV, SYM, 2>(ts, vt, N, c, stride_of(g, 2), ok[2], ok[D + 2], dinv, gr, gc);
     sinv = __ldg(vt + (long long)D * N + c);
   }
   pdl_wait();
@@ -292,7 +289,7 @@ __global__ void __launch_bounds__(32 * (2 * D + 1) * NS) k_st_colour(Grid g, int
       in = in && ir[k] >= 1 && ir[k] < g.n[k];
     }
     sp[row][part][lane] =
-        in ? row_share<T, TT, D, LV, SYM, NS>(g, ts, cr, ir, x, row < 2 * D ? k : D, part) : czero<Cx>();
+        in ? row_share<T, TT, LV, SYM, NS>(g, ts, cr, ir, x, row < 2 * D ? k : D, part) : czero<Cx>();
   }
   __syncthreads();
   if (wid || !live) return;
@@ -428,7 +425,7 @@ void colour_t(const Grid& g, int items, int nrhs, const TT* tab, const float2* v
   constexpr int NS = Ns<2>::colour;
   const int nit = (int)sel_items(items);
   const dim3 gr((unsigned)((g.ncell / 2 + 31) / 32) * nit);
-  launch_pdl(gr, 32 * 5 * NS, 0, s, k_st_colour<float, TT, 2, LV, SYM, NS>, g, nit, nrhs, tab, vt, wu, wp, colour, b, xi, xo,
+  launch_pdl(gr, 32 * 5 * NS, 0, s, k_st_colour<float, TT, LV, SYM, NS>, g, nit, nrhs, tab, vt, wu, wp, colour, b, xi, xo,
                                                                     g_sel.list);
 }
 template <typename T, typename TT, bool SYM>
