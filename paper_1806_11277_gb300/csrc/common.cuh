@@ -39,6 +39,18 @@ template <typename C> EHS_HD C czero() { C z; z.x = 0; z.y = 0; return z; }
 // 1 / z
 EHS_HD float2 cinv(float2 z) { float s = 1.0f / (z.x * z.x + z.y * z.y); return make_float2(z.x * s, -z.y * s); }
 EHS_HD double2 cinv(double2 z) { double s = 1.0 / (z.x * z.x + z.y * z.y); return make_double2(z.x * s, -z.y * s); }
+#ifdef __CUDACC__
+// z 2^e; on the exponent field where operand and result are normal numbers (no FP64 instruction)
+__device__ __forceinline__ double pow2_scaled(double x, int e) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  if (ex != 0 && ex != 0x7ff && ex + e > 0 && ex + e < 0x7ff)
+    return __hiloint2double(hi + (int)((unsigned)e << 20), __double2loint(x));
+  return ldexp(x, e);
+}
+__device__ __forceinline__ double2 pow2_scaled(double2 z, int e) {
+  return make_double2(pow2_scaled(z.x, e), pow2_scaled(z.y, e));
+}
+#endif
 EHS_HD float2 to_c(float2 z, float) { return z; }
 EHS_HD float2 to_c(double2 z, float) { return make_float2((float)z.x, (float)z.y); }
 EHS_HD double2 to_c(float2 z, double) { return make_double2(z.x, z.y); }

@@ -23,8 +23,6 @@
 namespace ehs {
 namespace {
 
-// x 2^e
-__device__ __forceinline__ double2 scaled(double2 v, int e) { return make_double2(ldexp(v.x, e), ldexp(v.y, e)); }
 // floor(log2 of the larger part), NONE for zero (and what is below the normal range)
 constexpr int NONE = -8192;
 __device__ __forceinline__ int exponent(double2 v) {
@@ -105,7 +103,7 @@ __global__ void k_dense_assemble(Grid g, StencilLayout L, const double2* __restr
           for (int k = 0; k < 3; ++k) in = in && j[k] >= 0 && j[k] < g.n[k];
           if (!in || !slot_valid(P.b, D, j)) continue;
           const long long col = (long long)P.b * g.ncell + cell_index(g, j);
-          const double2 v = scaled(ts[(long long)s * g.ncell + c], es[r] + es[col]);
+          const double2 v = pow2_scaled(ts[(long long)s * g.ncell + c], es[r] + es[col]);
           row[col].x += v.x;
           row[col].y += v.y;
         }
@@ -182,7 +180,7 @@ __global__ void k_dense_assemble_sub(Grid g, StencilLayout L, const double2* __r
           const long long gc = (long long)P.b * g.ncell + cell_index(g, j);
           const int lc = gl[gc];
           if (lc < 0) continue;
-          const double2 v = scaled(ts[(long long)sl * g.ncell + c], es[gs] + es[gc]);
+          const double2 v = pow2_scaled(ts[(long long)sl * g.ncell + c], es[gs] + es[gc]);
           row[lc].x += v.x;
           row[lc].y += v.y;
         }

@@ -469,8 +469,7 @@ __global__ void k_inv_columns(int N, const double2* __restrict__ A, const int* _
   const long long o = ((long long)mat * N + i) * N;
   const int* es = ex + (long long)mat * N;
   const int p = perm[(long long)mat * N + j], e = es[i] + es[p];
-  const double2 v = A[o + j];
-  X[o + p] = make_double2(ldexp(v.x, e), ldexp(v.y, e));
+  X[o + p] = pow2_scaled(A[o + j], e);
 }
 
 struct Plan {
@@ -508,7 +507,8 @@ template <int B> int clusters_of(int cl, size_t sm) {   // clusters of cl CTAs t
 // B = 32 columns a block up to N = 3200, else 16 (the panel's FP64 work halves, the update's passes over A double).
 // The panel is bound by the FP64 pipe of its SMs, so the cluster size is the one with the fewest rows per CTA
 // times waves of clusters, at one CTA per SM (at least 110 KB of shared memory each beside 9 to 17 KB of fixed arrays:
-// two to an SM, as clusters of 8 with 90 KB were placed, share its pipe).  GB300 runs 7 clusters of 16, 15 of 8, 23 of 6 or 36 of 4 that way.
+// two to an SM, as clusters of 8 with 90 KB were placed, share its pipe).  GB300 runs 7 clusters of 16, 15 of 8, 23 of
+// 6 or 36 of 4 that way.
 // 16 matrices of 1408: 455 us a block with clusters of 8, two to an SM; 511 with 15 of the 16 at a time; 339 with 6.
 Plan plan_for(int N, int nmat) {
   Plan p;
